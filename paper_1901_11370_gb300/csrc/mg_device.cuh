@@ -123,6 +123,28 @@ static void launch_coop(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStrea
     }
 }
 
+// One launch of thread-block clusters of `grid` CTAs; a refused launch is
+// kept for check_cuda like launch_k's.
+template <class... KArgs, class... Args>
+static void launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {grid.x, 1, 1};
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, ((KArgs)args)...);
+    if (e != cudaSuccess) {
+        int none = 0;
+        if (g_launch_error.compare_exchange_strong(none, (int)e))
+            g_launch_fail = {(const void *)kern, grid.x, block.x, smem};
+    }
+}
+
 // Quotient for the operator's coefficients and the Gauss-Seidel update: the
 // FP32 smoother (an inner solver under FP64 defect correction) takes the
 // fast reciprocal-based intrinsic; FP64 keeps the correctly rounded division.

@@ -168,6 +168,41 @@ struct LevelHost {
     std::vector<int> parents;  // segments holding the parents of its blocks
 };
 
+// Plan of the cluster kernel that runs the levels 0 .. top of a cycle
+// (mg_bottom.cu): the cut of each level into slabs, the shared-memory
+// layout of a CTA, and where the top level lives in the pool.
+constexpr int kBotMaxLev = 8;
+struct BotPlan {
+    int top = 0;                    // highest level of the kernel (0: no plan)
+    int n0[3];                      // cells of level 0 in the local dimensions a, b, p
+    int perm[3];                    // original dimension of a, b, p (2D: b = 2)
+    int PB, PP;                     // CTAs along b and p
+    int mb, mp;                     // largest slab of level 0 along b and p
+    int array0;                     // bytes before the field arrays (coarsest residual)
+    int offx[kBotMaxLev], offf[kBotMaxLev], offv[kBotMaxLev], offj;  // element offsets: x, f, v_old per level, Jacobi copy
+    int dn[kBotMaxLev], up[kBotMaxLev];                              // smoothing steps
+    long long woff[kBotMaxLev];     // dense coefficients of a level
+    int n, nblk[3], nref;           // top level: block size, blocks per dimension, covered blocks
+    long long cell_first, ghost_first;
+    const int *bmap, *bmap0;        // block coordinates -> index within the level (top level, level 0)
+    int cn, cnblk[3];               // level 0: block size, blocks per dimension
+    int nc, ns, singular;
+    int fmg, jac;
+    int fd;                         // 1: coarsest solve by eigenvectors (constant eps)
+    const double *fdtab;            // eigenvectors along a, along b ([cell][mode]), then the solves along p ([p'][p][kb][ka])
+};
+struct BotState {                   // one per precision and smoother
+    bool tried = false;
+    BotPlan plan;
+    size_t smem = 0;
+    int *d_map = nullptr;           // block maps of levels 0 .. top
+    long long mapoff[kBotMaxLev];
+    void *d_w = nullptr;            // dense coefficients (variable eps), the kernel's precision
+    double *d_w0 = nullptr;         // those of level 0 in FP64 (coarsest residual)
+    double *d_fd = nullptr;         // tables of the eigenvector solve (BotPlan::fdtab)
+    long long wtotal = 0;
+};
+
 }  // namespace mg
 
 struct mg_tree {
@@ -271,6 +306,12 @@ struct mg_tree {
     // a tree made by adapt: sweep variants by level depth taken over from the
     // old tree instead of autotuning (per precision; empty: tune)
     std::map<int, int> tune_hint[2];
+    // cluster kernel of the lower levels (mg_bottom.cu): its plans per
+    // precision and smoother; whether the running call uses it (the solve
+    // loops do); precisions whose sweep kernels the caller has pinned
+    mg::BotState bottom[2][2];
+    bool bottom_on = false;
+    bool pinned[2] = {false, false};
 };
 
 namespace mg {
@@ -314,6 +355,12 @@ void widen_f64(mg_tree *t, const float *a, double *b, long long n);
 // FP64 face coefficients of every cell into t->d_wface (eps ghosts current)
 void face_coef(mg_tree *t);
 KParams kparams(mg_tree *t, int homog);
+// the lower levels in one launch (mg_bottom.cu)
+template <class T> int bottom_level(mg_tree *t);
+template <class T> void bottom_prepare(mg_tree *t);
+template <class T> void bottom_run(mg_tree *t, const KParams &P, Fields<T> &F, bool fmg, int nd, int nu);
+void bottom_coef(mg_tree *t);
+void bottom_free(mg_tree *t);
 int time_sweeps(mg_tree *t, int level, int n_sweeps, int prec, double *out4);
 // batch: per-tree composite residual sums (3 per tree, on the host after wait)
 void residual_enqueue_trees(mg_tree *t, Fields<double> &F, float *f32_cells, bool want_max,

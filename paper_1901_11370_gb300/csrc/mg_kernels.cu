@@ -4329,7 +4329,8 @@ template <class T, int D> struct Launch {
     // Downward FAS step from group g to g-1 (Sec. 2.4): every non-coarsest
     // segment of g restricts into its parents (pushing the parent-level
     // ghosts), then f^H and v_old are formed on the covered blocks of g-1.
-    static void restrict_group(mg_tree *t, const KParams &P, int g, Fields<T> &F) {
+    // no_fas: the covered blocks of g-1 are left to the cluster kernel (mg_bottom.cu).
+    static void restrict_group(mg_tree *t, const KParams &P, int g, Fields<T> &F, bool no_fas = false) {
         // parent segments fed by a restriction without ghost push get a
         // ghost fill before their FAS right-hand side
         std::vector<char> plain(t->lev.size(), 0);
@@ -4365,6 +4366,7 @@ template <class T, int D> struct Launch {
             }
         }
         if (!flat.empty()) restrict_flat(t, P, flat, F.X, F.XG, F.F, F.E, F.EG, F.F, 1);
+        if (no_fas) return;
         std::vector<int> flat_ghost, flat_fas;
         for (int c : t->groups[g - 1])
             if (plain[c]) {
@@ -4537,6 +4539,19 @@ template <class T, int D> struct Launch {
     // ghosts and the upward steps up to the cut in another.
     static void vcycle(mg_tree *t, Fields<T> &F, int top, int nd, int nu, int homog, int strict = 0) {
         const KParams P = kparams(t, homog);
+        const int bot = std::min(bottom_level<T>(t), top);
+        if (bot > 0) {  // levels 0 .. bot in one launch
+            for (int g = top; g > bot; g--) {
+                smooth_group(t, P, g, F, nd, true);
+                restrict_group(t, P, g, F, g - 1 == bot);
+            }
+            bottom_run<T>(t, P, F, false, nd, nu);
+            for (int g = bot + 1; g <= top; g++) {
+                prolong_group(t, P, g, F);
+                smooth_group(t, P, g, F, nu, false);
+            }
+            return;
+        }
         const int cut = tail_cut(t, top);
         TailRec tr;
         tr.P = P;
@@ -4560,6 +4575,16 @@ template <class T, int D> struct Launch {
     static void fmg(mg_tree *t, Fields<T> &F, int nd, int nu, int homog) {
         const KParams P = kparams(t, homog);
         const int top = (int)t->groups.size() - 1;
+        const int bot = bottom_level<T>(t);
+        if (bot > 0) {
+            for (int g = top; g > bot; g--) restrict_group(t, P, g, F, g - 1 == bot);
+            bottom_run<T>(t, P, F, true, nd, nu);
+            for (int g = bot + 1; g <= top; g++) {
+                prolong_group(t, P, g, F);
+                vcycle(t, F, g, nd, nu, homog, 1);
+            }
+            return;
+        }
         const int cut = tail_cut(t, top);
         TailRec tr;
         tr.P = P;

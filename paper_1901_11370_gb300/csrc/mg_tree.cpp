@@ -1119,7 +1119,10 @@ extern "C" int mg_set_eps(mg_tree *t, const double *e) {
     if (!e) return fail(MG_ERR_ARG, "null eps");
     int rc;
     if ((rc = dalloc(&t->f64.E, t->ncells)) || (rc = dalloc(&t->f64.EG, t->nghost))) return rc;
-    if (!t->var_eps) drop_graphs(t);  // eps pointers enter the captured kernels
+    if (!t->var_eps) {  // eps pointers enter the captured kernels; the cluster kernel's coarsest solve changes
+        drop_graphs(t);
+        bottom_free(t);
+    }
     t->var_eps = true;
     if ((rc = leaf_copy(t, t->f64.E, e, true))) return rc;
     refresh_eps<double>(t, t->f64);
@@ -1129,6 +1132,7 @@ extern "C" int mg_set_eps(mg_tree *t, const double *e) {
     t->adj.E = t->f64.E;
     t->adj.W = t->f64.W;
     t->adj.EG = t->f64.EG;
+    bottom_coef(t);
     if (t->f32.X) {
         if ((rc = dalloc(&t->f32.E, t->ncells)) || (rc = dalloc(&t->f32.EG, t->nghost))) return rc;
         copy_eps_to_f32(t);
@@ -1201,6 +1205,16 @@ static int use_params(mg_tree *t, const mg_params *p, mg_params *q, std::string 
     return MG_OK;
 }
 
+// The solve loops run the lower levels in one cluster launch per cycle;
+// mg_vcycle and mg_fmg keep the launch-by-launch cycle, which the sweep
+// variants and the tail option are defined on.
+struct BottomScope {
+    mg_tree *t;
+    bool was;
+    explicit BottomScope(mg_tree *tree) : t(tree), was(tree->bottom_on) { t->bottom_on = true; }
+    ~BottomScope() { t->bottom_on = was; }
+};
+
 extern "C" int mg_vcycle(mg_tree *t, int n, const mg_params *p) {
     NEED_FINAL(t);
     mg_params q;
@@ -1256,6 +1270,7 @@ static int ensure_f32(mg_tree *t) {
 extern "C" int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_first, const mg_params *p,
                         int *cycles_done, double *rel_out) {
     NEED_FINAL(t);
+    BottomScope scope(t);
     mg_params q;
     std::string sfx;
     int rc;
@@ -1280,6 +1295,7 @@ extern "C" int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_firs
     // each step is one graph: the cycle(s) and the FP64 composite residual,
     // whose norms arrive in pinned host memory; the host only waits
     if (q.precision == MG_FP64) {
+        bottom_prepare<double>(t);
         if ((rc = run_graph(t, "res64", [&] { residual_enqueue(t, t->f64, 0, nullptr, nullptr); }))) return rc;
         residual_wait(t, o);
         const double r0 = std::sqrt(o[0] / o[1]);
@@ -1307,6 +1323,7 @@ extern "C" int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_firs
         }
     } else if (q.precision == MG_FP32_DC) {
         if ((rc = ensure_f32(t))) return rc;
+        bottom_prepare<float>(t);
         if ((rc = run_graph(t, "res64f32", [&] { residual_enqueue(t, t->f64, 0, nullptr, t->f32.F); }))) return rc;
         residual_wait(t, o);
         const double r0 = std::sqrt(o[0] / o[1]);
@@ -1378,6 +1395,8 @@ static int adjoint_setup(mg_tree *t, const mg_params *p, mg_params *q) {
     t->adj.E = t->f64.E;
     t->adj.W = t->f64.W;
     t->adj.EG = t->f64.EG;
+    bottom_prepare<double>(t);
+    if (q->precision == MG_FP32_DC) bottom_prepare<float>(t);
     return adjoint_buffers(t);
 }
 
@@ -1386,6 +1405,7 @@ static int adjoint_run(mg_tree *t, const double *g, double *dLdf, double *dLdeps
     NEED_FINAL(t);
     if (!g || !dLdf) return fail(MG_ERR_ARG, "null argument");
     if (max_cycles < 0) return fail(MG_ERR_ARG, "negative cycle count");
+    BottomScope scope(t);
     mg_params q;
     int rc, it = 0;
     double rel = 0.0;
@@ -1428,6 +1448,7 @@ extern "C" int mg_clean_adjoint(mg_tree *t, const double *gBnew, double *gB, con
     if (!gBnew || !gB || gBnew == gB) return fail(MG_ERR_ARG, "null or aliased argument");
     if (t->geom != MG_CART) return fail(MG_ERR_UNSUPPORTED, "divergence cleaning: Cartesian meshes only");
     if (!(rel_tol > 0) || max_cycles < 0) return fail(MG_ERR_ARG, "rel_tol must be positive, max_cycles >= 0");
+    BottomScope scope(t);
     mg_params q;
     int rc, it = 0;
     double rel = 0.0;
@@ -1623,6 +1644,7 @@ extern "C" int mg_set_sweep_variant(mg_tree *t, int precision, int level, int va
         if (variant < 0) ch[l] = -1;
         else if (sweep_variant_ok(t, prec, l, variant)) ch[l] = variant;
     }
+    t->pinned[prec] = variant >= 0 || (level >= 0 && t->pinned[prec]);  // pinned levels run their own sweeps
     drop_graphs(t);  // captured cycles hold the previous choice
     return MG_OK;
 }
@@ -1690,6 +1712,7 @@ extern "C" int mg_tree_destroy(mg_tree *t) {
         free_fields(t->f64, true);
         free_fields(t->adj, false);
         free_fields(t->f32, true);
+        bottom_free(t);
         cudaFree(t->d_blocks); cudaFree(t->d_levels); cudaFree(t->d_bcplanes);
         cudaFree(t->d_r64); cudaFree(t->d_wface); cudaFree(t->d_jac64); cudaFree(t->d_jac32); cudaFree(t->d_minv); cudaFree(t->d_cvec); cudaFree(t->d_partials); cudaFree(t->d_red); cudaFree(t->d_status); cudaFree(t->d_tcoarse); cudaFree(t->d_coarse_chunks);
         cudaFree(t->d_bt); cudaFree(t->d_bt32); cudaFree(t->d_btperm); cudaFree(t->d_btlist); cudaFree(t->d_bt_chunks);
