@@ -315,12 +315,14 @@ __global__ void __launch_bounds__(256) k_adj_vec(KParams P, int first, long long
     }
 }
 
-// Sum of n partial pairs (one CTA, fixed order: deterministic).
-__global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict__ partials, int n,
-                                                       double *__restrict__ out) {
+// Sum of n partial pairs (one CTA, fixed order: deterministic).  Eight
+// warps and two shuffle stages, as in the residual norms' reduction.
+constexpr int kSumThreads = 256;
+__global__ void __launch_bounds__(kSumThreads) k_sum_partials(const double *__restrict__ partials, int n,
+                                                              double *__restrict__ out) {
     pdl_entry();
     double a = 0, z = 0;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    for (int e = threadIdx.x; e < n; e += kSumThreads) {
         a += partials[3 * e];
         z += partials[3 * e + 1];
     }
@@ -328,15 +330,21 @@ __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict_
         a += __shfl_down_sync(0xffffffffu, a, o);
         z += __shfl_down_sync(0xffffffffu, z, o);
     }
-    __shared__ double sh[2][32];
+    constexpr int NW = kSumThreads / 32;
+    __shared__ double sh[2][NW];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) { sh[0][w] = a; sh[1][w] = z; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double x = 0, y = 0;
-        for (int e = 0; e < (int)(blockDim.x >> 5); e++) { x += sh[0][e]; y += sh[1][e]; }
-        out[0] = x;
-        out[1] = y;
+    if (w) return;
+    a = lane < NW ? sh[0][lane] : 0.0;
+    z = lane < NW ? sh[1][lane] : 0.0;
+    for (int o = NW / 2; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        z += __shfl_down_sync(0xffffffffu, z, o);
+    }
+    if (lane == 0) {
+        out[0] = a;
+        out[1] = z;
     }
 }
 
@@ -425,8 +433,7 @@ template <int D> struct Adj {
         }
         if (!sums) return;
         ++t->launches;
-        launch_k(k_sum_partials, 1, 1024, 0, t->stream, (const double *)t->d_partials, slot, t->d_red);
-        cudaMemcpyAsync(t->h_red, t->d_red, 2 * sizeof(double), cudaMemcpyDeviceToHost, t->stream);
+        launch_k(k_sum_partials, 1, kSumThreads, 0, t->stream, (const double *)t->d_partials, slot, t->h_red);  // pinned
         cudaStreamSynchronize(t->stream);
         sums[0] = t->h_red[0];
         sums[1] = t->h_red[1];

@@ -273,8 +273,7 @@ struct mg_tree {
     double *d_cvec = nullptr;      // coarsest residual vector (ns)
     double *d_partials = nullptr;  // per-CTA norm partials (3 per CTA)
     int n_partials = 0;
-    double *d_red = nullptr;       // reduced norms (3)
-    double *h_red = nullptr;       // pinned host copy
+    double *h_red = nullptr;       // reduced norms (3), pinned: the reductions write here
     long long launches = 0;        // kernels launched so far
     int *d_status = nullptr;       // device status word (0 = ok), then the tail kernel's grid-barrier
                                    // counter and generation (kStatusWords ints, cleared together)

