@@ -271,6 +271,8 @@ struct mg_tree {
     int nc = 0, ns = 0;            // coarsest cells, system size (nc + singular) -- one tree
     bool minv_ok = false;
     double *d_cvec = nullptr;      // coarsest residual vector (ns)
+    double *d_cwork = nullptr;     // work of the device inverse (mg_coarse.cu)
+    int *d_crow = nullptr, *d_cflag = nullptr;  // its cell -> row map and status
     double *d_partials = nullptr;  // per-CTA norm partials (3 per CTA)
     int n_partials = 0;
     double *h_red = nullptr;       // reduced norms (3), pinned: the reductions write here
@@ -354,6 +356,9 @@ void widen_f64(mg_tree *t, const float *a, double *b, long long n);
 // FP64 face coefficients of every cell into t->d_wface (eps ghosts current)
 void face_coef(mg_tree *t);
 KParams kparams(mg_tree *t, int homog);
+// dense inverse of a single tree's coarsest level on the device (mg_coarse.cu):
+// 0 done, 1 left to the host, < 0 an error
+int coarse_inverse_device(mg_tree *t);
 // the lower levels in one launch (mg_bottom.cu)
 template <class T> int bottom_level(mg_tree *t);
 template <class T> void bottom_prepare(mg_tree *t);

@@ -704,9 +704,15 @@ static void coarse_plan(const mg_tree *src, TreeCoarse &tc, const LevelHost &L, 
     tc.bt_P = tc.nc / tc.bt_n;
 }
 
-// Coarsest-level factors of every tree (trees in parallel host threads):
+// Coarsest-level factors: a single tree's dense inverse on the device
+// (mg_coarse.cu); else of every tree (trees in parallel host threads):
 // dense inverses, and plane records of the block-tridiagonal trees.
 int build_coarse_inverse(mg_tree *t) {
+    const int dev = coarse_inverse_device(t);
+    if (dev <= 0) {
+        t->minv_ok = dev == 0;
+        return dev;
+    }
     std::vector<double> eps;
     if (t->var_eps) {
         CK(cudaStreamSynchronize(t->stream));
@@ -1713,7 +1719,7 @@ extern "C" int mg_tree_destroy(mg_tree *t) {
         free_fields(t->f32, true);
         bottom_free(t);
         cudaFree(t->d_blocks); cudaFree(t->d_levels); cudaFree(t->d_bcplanes);
-        cudaFree(t->d_r64); cudaFree(t->d_wface); cudaFree(t->d_jac64); cudaFree(t->d_jac32); cudaFree(t->d_minv); cudaFree(t->d_cvec); cudaFree(t->d_partials); cudaFree(t->d_status); cudaFree(t->d_tcoarse); cudaFree(t->d_coarse_chunks);
+        cudaFree(t->d_r64); cudaFree(t->d_wface); cudaFree(t->d_jac64); cudaFree(t->d_jac32); cudaFree(t->d_minv); cudaFree(t->d_cvec); cudaFree(t->d_cwork); cudaFree(t->d_crow); cudaFree(t->d_cflag); cudaFree(t->d_partials); cudaFree(t->d_status); cudaFree(t->d_tcoarse); cudaFree(t->d_coarse_chunks);
         cudaFree(t->d_bt); cudaFree(t->d_bt32); cudaFree(t->d_btperm); cudaFree(t->d_btlist); cudaFree(t->d_bt_chunks);
         cudaFreeHost(t->h_red);
         cudaFree(t->d_runs); cudaFree(t->d_slot_off); cudaFree(t->d_slots); cudaFree(t->d_tree3);
