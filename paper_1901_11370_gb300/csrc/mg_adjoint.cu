@@ -87,7 +87,8 @@ __device__ __forceinline__ double *addr(double *A, double *AG, const BlockDesc &
 // Step 1 on the leaf blocks [first, first + gridDim.x) of one level.  Y is
 // the leaf-order input (kind T_GRAD: dim arrays of nleaf values).  Writes
 // the adjoint of every interior cell (A) and of every ghost slot a row of
-// this block reads (AG); the caller zeroes AG first.
+// this block reads (AG); the caller zeroes AG first.  W: the operator's
+// precomputed coefficients (variable eps or the cylindrical form), else null.
 //   T_OPERATOR: rows sum_f w_f (x_nb - x_c) - lambda x_c of A (Sec. 2.2);
 //   T_EPS:      y = lambda, the rows' derivative -y d(w_f)/d eps with the
 //               harmonic mean w_f ~ 2 e_c e_o / (e_c + e_o) and phi = X;
@@ -99,7 +100,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_stencil_T(KParams P, int first,
                                                            long long nleaf, const double *__restrict__ X,
                                                            const double *__restrict__ XG,
                                                            const double *__restrict__ E,
-                                                           const double *__restrict__ EG, double *__restrict__ A,
+                                                           const double *__restrict__ EG,
+                                                           const double *__restrict__ W, double *__restrict__ A,
                                                            double *__restrict__ AG) {
     pdl_entry();
     __shared__ BlockDesc sb;
@@ -113,7 +115,27 @@ __global__ void __launch_bounds__(kMaxThreads) k_stencil_T(KParams P, int first,
         cell_of(c, n, D, i, j, k);
         const I3 p{i, j, k};
         double acc = 0.0;
-        if (kind == T_OPERATOR) {
+        if (kind == T_OPERATOR && (W || (!E && P.geom == MG_CART))) {
+            // weights read, not formed: with variable eps the form below takes
+            // twelve FP64 divisions a cell (about ten instructions each)
+            const double yc = y[c];
+            const double *ws = W ? W + b.cell_off * wstride(D) : nullptr;
+            acc = -(W ? ws[2 * D * C + c] : L.diag) * yc;
+#pragma unroll
+            for (int d = 0; d < D; d++)
+#pragma unroll
+                for (int s = 0; s < 2; s++) {
+                    I3 q = p;
+                    const int qd = get(p, d) + (s ? 1 : -1);
+                    put(q, d, qd);
+                    if (qd >= 0 && qd < n) {
+                        const int cq = cidx<D>(n, q.x, q.y, q.z);
+                        acc = fma(W ? ws[(2 * d + 1 - s) * C + cq] : L.inv_h2[d], y[cq], acc);
+                    } else {
+                        AG[b.ghost_off + (2 * d + s) * F + tidx<D>(n, d, i, j, k)] = (W ? ws[(2 * d + s) * C + c] : L.inv_h2[d]) * yc;
+                    }
+                }
+        } else if (kind == T_OPERATOR) {
             double sw = 0.0;
             const double yc = y[c];
 #pragma unroll
@@ -398,7 +420,8 @@ template <int D> struct Adj {
             if (nleaf <= 0) continue;
             ++t->launches;
             launch_k(k_stencil_T<D>, nleaf, threads_of(cells_of<D>(L.n)), 0, t->stream, P, L.first + L.nref, kind,
-                     dc, Y, leaf_base, (long long)t->nleaf_cells, X, XG, E, EG, t->d_at, t->d_atg);
+                     dc, Y, leaf_base, (long long)t->nleaf_cells, X, XG, E, EG, (const double *)t->f64.W, t->d_at,
+                     t->d_atg);
             leaf_base += (long long)nleaf * cells_of<D>(L.n);
         }
     }
