@@ -2070,7 +2070,6 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
             rs[c] = fs[c] - (lap - kp_helm<T>(P) * xc);
         }
         __syncthreads();
-        const int pn = p.n;
         for (int c = tid; c < M; c += nth) {
             const int ci = c % m, cj = (c / m) % m, ck = D == 3 ? c / (m * m) : 0;
             T sx = 0, sr = 0;
@@ -2103,6 +2102,44 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
             I3 ii = face_cell<D>(m, face, v, false);
             ii.x += b.poff[0];
             ii.y += b.poff[1];
+        const int pn = p.n;
+        bool done = false;
+        if constexpr (sizeof(T) == 8) {
+            // FP64, constant coefficient: the Laplacians of the 2^D children
+            // of a parent cell share their inner faces, whose fluxes cancel.
+            // What is left is sum_d w_d (outer neighbours in d - children):
+            // 5 instead of 16 FP64 instructions a child in 3D, and no pass
+            // over the child residuals (128^3 Jacobi solve: 44 -> 20 us a launch).
+            if (!var && !cyl) {
+                done = true;
+                const T wsum = ih0 + ih1 + (D == 3 ? ih2 : (T)0) + kp_helm<T>(P), inv = (T)(1.0 / (1 << D));
+                for (int c = tid; c < M; c += nth) {
+                    const int ci = c % m, cj = (c / m) % m, ck = D == 3 ? c / (m * m) : 0;
+                    T sx = 0, sf = 0, ox = 0, oy = 0, oz = 0;
+#pragma unroll
+                    for (int g = 0; g < (D == 3 ? 2 : 1); g++)
+#pragma unroll
+                        for (int e = 0; e < 2; e++) {  // the row of two children at j + e, k + g
+                            const int i = 2 * ci, j = 2 * cj + e, k = D == 3 ? 2 * ck + g : 0, fc = cidx<D>(n, i, j, k);
+                            sx += xs[fc] + xs[fc + 1];
+                            sf += fs[fc] + fs[fc + 1];
+                            ox += nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i + 1, j, k, 0, 1);
+                            oy += nbv(xs, gs, i, j, k, 1, e) + nbv(xs, gs, i + 1, j, k, 1, e);
+                            if (D == 3) oz += nbv(xs, gs, i, j, k, 2, g) + nbv(xs, gs, i + 1, j, k, 2, g);
+                        }
+                    T r = fma(wsum, sx, sf);
+                    r = fma(-ih0, ox, r);
+                    r = fma(-ih1, oy, r);
+                    if (D == 3) r = fma(-ih2, oz, r);
+                    const T xv = sx * inv;
+                    const int pc = cidx<D>(pn, b.poff[0] + ci, b.poff[1] + cj, b.poff[2] + ck);
+                    F.X[p.cell_off + pc] = xv;
+                    F.F[p.cell_off + pc] = r * inv;
+                    rs[c] = xv;
+                }
+            }
+        }
+        if (!done) {
             ii.z += D == 3 ? b.poff[2] : 0;
             put(ii, d, s ? pn - 1 : 0);
             int u;
@@ -2155,6 +2192,7 @@ __global__ void __launch_bounds__(128) k_restrict_rows(KParams P, int first, int
         }
     };
     auto parent = [&](int g, Src &r) {
+        }
         if (g < nblocks) r.plev = P.B[r.par].lev;
     };
     auto issue = [&](int it, int g, const Src &r) {  // thread ISSUER only
@@ -2219,26 +2257,55 @@ __global__ void __launch_bounds__(128) k_restrict_rows(KParams P, int first, int
         ld4(xs + 8 * r + 4 * h, xr + 1);
         xr[0] = h ? xs[8 * r + 3] : gs[j + 8 * k];
         xr[5] = h ? gs[FC + j + 8 * k] : xs[8 * r + 4];
-        ld4(j > 0 ? xs + 8 * (r - 1) + 4 * h : gs + 2 * FC + 4 * h + 8 * k, dn);
-        ld4(j < n - 1 ? xs + 8 * (r + 1) + 4 * h : gs + 3 * FC + 4 * h + 8 * k, up);
-        ld4(k > 0 ? xs + 8 * (r - 8) + 4 * h : gs + 4 * FC + 4 * h + 8 * j, bk);
-        ld4(k < n - 1 ? xs + 8 * (r + 8) + 4 * h : gs + 5 * FC + 4 * h + 8 * j, fw);
+        T oy[4], oz[4];  // FP64: the neighbour rows outside the 2x2x2 children
+        if constexpr (sizeof(T) == 8) {
+            const bool jo = j & 1, ko = k & 1;
+            ld4(jo ? (j < n - 1 ? xs + 8 * (r + 1) + 4 * h : gs + 3 * FC + 4 * h + 8 * k)
+                   : (j > 0 ? xs + 8 * (r - 1) + 4 * h : gs + 2 * FC + 4 * h + 8 * k), oy);
+            ld4(ko ? (k < n - 1 ? xs + 8 * (r + 8) + 4 * h : gs + 5 * FC + 4 * h + 8 * j)
+                   : (k > 0 ? xs + 8 * (r - 8) + 4 * h : gs + 4 * FC + 4 * h + 8 * j), oz);
+        } else {
+            ld4(j > 0 ? xs + 8 * (r - 1) + 4 * h : gs + 2 * FC + 4 * h + 8 * k, dn);
+            ld4(j < n - 1 ? xs + 8 * (r + 1) + 4 * h : gs + 3 * FC + 4 * h + 8 * k, up);
+            ld4(k > 0 ? xs + 8 * (r - 8) + 4 * h : gs + 4 * FC + 4 * h + 8 * j, bk);
+            ld4(k < n - 1 ? xs + 8 * (r + 8) + 4 * h : gs + 5 * FC + 4 * h + 8 * j, fw);
+        }
         ld4(fs + 8 * r + 4 * h, f4);
-        T res[4];
+        T s4[4];
+        if constexpr (sizeof(T) == 8) {
+            // the inner faces of the 2x2x2 children cancel (see
+            // k_restrict_tma): of each row only the outer y and z neighbours
+            // and both ends of the cell pairs count.  26 instead of 68 FP64
+            // instructions a thread.
+            const T wsum = w0 + w1 + w2 + helm;
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const T xc = xr[1 + q];
-            T lap = 0;
-            lap += w0 * (xr[q] - xc);
-            lap += w0 * (xr[q + 2] - xc);
-            lap += w1 * (dn[q] - xc);
-            lap += w1 * (up[q] - xc);
-            lap += w2 * (bk[q] - xc);
-            lap += w2 * (fw[q] - xc);
-            res[q] = f4[q] - (lap - helm * xc);
+            for (int q = 0; q < 2; q++) {
+                s4[q] = xr[1 + 2 * q] + xr[2 + 2 * q];
+                T rr = fma(wsum, s4[q], f4[2 * q] + f4[2 * q + 1]);
+                rr = fma(-w0, xr[2 * q] + xr[3 + 2 * q], rr);
+                rr = fma(-w1, oy[2 * q] + oy[2 * q + 1], rr);
+                s4[2 + q] = fma(-w2, oz[2 * q] + oz[2 * q + 1], rr);
+            }
+        } else {
+            T res[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const T xc = xr[1 + q];
+                T lap = 0;
+                lap += w0 * (xr[q] - xc);
+                lap += w0 * (xr[q + 2] - xc);
+                lap += w1 * (dn[q] - xc);
+                lap += w1 * (up[q] - xc);
+                lap += w2 * (bk[q] - xc);
+                lap += w2 * (fw[q] - xc);
+                res[q] = f4[q] - (lap - helm * xc);
+            }
+            s4[0] = xr[1] + xr[2];
+            s4[1] = xr[3] + xr[4];
+            s4[2] = res[0] + res[1];
+            s4[3] = res[2] + res[3];
         }
         // sums under parent cells 2h, 2h + 1: this row's pairs, then rows j ^ 1, k ^ 1
-        T s4[4] = {xr[1] + xr[2], xr[3] + xr[4], res[0] + res[1], res[2] + res[3]};
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             s4[q] += __shfl_xor_sync(0xffffffffu, s4[q], 2);
