@@ -157,6 +157,8 @@ template <class T> __device__ __forceinline__ T lv_ih(const LevelDesc &L, int d)
 template <> __device__ __forceinline__ float lv_ih<float>(const LevelDesc &L, int d) { return L.inv_h2f[d]; }
 template <class T> __device__ __forceinline__ T lv_idiag(const LevelDesc &L) { return (T)L.inv_diag; }
 template <> __device__ __forceinline__ float lv_idiag<float>(const LevelDesc &L) { return L.inv_diagf; }
+template <class T> __device__ __forceinline__ T lv_wd(const LevelDesc &L, int d) { return (T)L.wd[d]; }
+template <> __device__ __forceinline__ float lv_wd<float>(const LevelDesc &L, int d) { return L.inv_h2f[d] * L.inv_diagf; }
 template <class T> __device__ __forceinline__ T lv_h0(const LevelDesc &L) { return (T)L.h[0]; }
 template <> __device__ __forceinline__ float lv_h0<float>(const LevelDesc &L) { return L.h0f; }
 template <class T> __device__ __forceinline__ T kp_lo0(const KParams &P) { return (T)P.lo[0]; }

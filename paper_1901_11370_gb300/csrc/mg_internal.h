@@ -51,6 +51,8 @@ struct LevelDesc {
     double inv_diag;      // 1 / (2 sum_d 1/h_d^2 + lambda): constant-coefficient Gauss-Seidel divisor
     double diag;          // 2 sum_d 1/h_d^2 + lambda: the constant-coefficient row diagonal
     double vol;           // cell volume (Cartesian)
+    double wd[3];         // inv_h2 / diag: constant-coefficient Gauss-Seidel weights
+    double pad;
     // FP32 copies, so that FP32 kernels do no FP64 arithmetic or conversion
     float inv_h2f[3];
     float inv_diagf, h0f, hvf;  // 1/diag, h_0, 2 pi h_0 h_1 (cylindrical volume per unit r)

@@ -378,6 +378,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
+// The FP64 Gauss-Seidel value of a constant-coefficient cell from its three
+// neighbour sums, 1 / diagonal multiplied into the weights on the host: one
+// product and D FMAs after the sums, against a product, two FMAs, a
+// subtraction and a product -- 7 instead of 8 FP64 instructions a cell in 3D.
+// GB300's FP64 unit bounds these sweeps (finest level of the 19.8M-cell
+// tree: 6.2M cells x 8 at 5.9e11 / s is 84 us).
+template <int D> __device__ __forceinline__ double gs_const64(const LevelDesc &L, double sx, double sy, double sz, double f) {
+    double v = fma(L.wd[0], sx, -f * L.inv_diag);
+    v = fma(L.wd[1], sy, v);
+    return D == 3 ? fma(L.wd[2], sz, v) : v;
+}
+
 // HALF: half as many threads per CTA (two colour cells each), which wastes
 // less at the CTA barriers on levels with few blocks per SM.
 template <class T, int D, int NT, bool HALF = false>
@@ -523,10 +535,16 @@ __global__ void __launch_bounds__(sweep_tma_threads(cells_of<D>(NT) / 2, HALF), 
             const int c = cidx<D>(n, i, j, k);
             T xnew;
             if (!var && !cyl) {
-                T num = w0 * (nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i, j, k, 0, 1)) +
-                        w1 * (nbv(xs, gs, i, j, k, 1, 0) + nbv(xs, gs, i, j, k, 1, 1));
-                if (D == 3) num += w2 * (nbv(xs, gs, i, j, k, 2, 0) + nbv(xs, gs, i, j, k, 2, 1));
-                xnew = (num - fs[c]) * inv_den;
+                const T sx = nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i, j, k, 0, 1);
+                const T sy = nbv(xs, gs, i, j, k, 1, 0) + nbv(xs, gs, i, j, k, 1, 1);
+                const T sz = D == 3 ? nbv(xs, gs, i, j, k, 2, 0) + nbv(xs, gs, i, j, k, 2, 1) : (T)0;
+                if constexpr (sizeof(T) == 8) {
+                    xnew = gs_const64<D>(L, sx, sy, sz, fs[c]);
+                } else {
+                    T num = w0 * sx + w1 * sy;
+                    if (D == 3) num += w2 * sz;
+                    xnew = (num - fs[c]) * inv_den;
+                }
             } else if (wc) {  // same terms and order as below, coefficients read, 1 / diagonal precomputed
                 const T *ws = es + c;
                 T num = ws[0] * nbv(xs, gs, i, j, k, 0, 0);
@@ -917,8 +935,13 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 8 ? ((FG && STAGES == 2) 
                 const T sy = p ? dn[o] + up[o] : dn[e] + up[e];
                 const T sz = p ? bk[o] + fw[o] : bk[e] + fw[e];
                 const T fv = p ? fr[o] : fr[e];
-                const T num = w0 * (xm + xp) + w1 * sy + w2 * sz;
-                const T xnew = (num - fv) * inv_den;
+                T xnew;
+                if constexpr (sizeof(T) == 8) {
+                    xnew = gs_const64<3>(L, xm + xp, sy, sz, fv);
+                } else {
+                    const T num = w0 * (xm + xp) + w1 * sy + w2 * sz;
+                    xnew = (num - fv) * inv_den;
+                }
                 newrow[h][e] = p ? r[e] : xnew;
                 newrow[h][o] = p ? xnew : r[o];
             }
@@ -1210,6 +1233,10 @@ __global__ void __launch_bounds__(kMaxThreads) k_fas_rhs_vold(KParams P, int fir
 // cell of block b changes, so after the correction all its face ghosts that
 // depend on its cells are pushed (the kernel reads only the coarser level's
 // fields and its own interior, never this level's ghosts).
+// Each difference x^H - x^H_old is formed once, into a box over the parent
+// cells under the block and their face halo: a cell then takes 4 FP64
+// instructions instead of 9 and four shared loads instead of eight global
+// ones (FP64 16^3 blocks, whose staged form does not fit: see prolong).
 template <class T, int D>
 __global__ void __launch_bounds__(kMaxThreads) k_prolong_push(KParams P, int first, Fields<T> F) {
     pdl_entry();
@@ -1221,19 +1248,24 @@ __global__ void __launch_bounds__(kMaxThreads) k_prolong_push(KParams P, int fir
     stage_desc(P, b.parent, sp);
     const BlockDesc &p = sp;
     const LevelDesc &L = P.L[b.lev];
-    const int n = b.n, C = cells_of<D>(n);
+    const int n = b.n, C = cells_of<D>(n), B = n / 2 + 2, BB = D == 3 ? B * B * B : B * B;
+    T *box = xs + C;
+    for (int q = threadIdx.x; q < BB; q += blockDim.x) {
+        const int a = q % B, c = (q / B) % B, e = D == 3 ? q / (B * B) : 1;
+        if ((a == 0 || a == B - 1) + (c == 0 || c == B - 1) + (D == 3 && (e == 0 || e == B - 1)) > 1) continue;  // never read
+        const int i = b.poff[0] + a - 1, j = b.poff[1] + c - 1, k = D == 3 ? b.poff[2] + e - 1 : 0;
+        box[q] = load<T, D>(F.X, F.XG, p, i, j, k) - load<T, D>(F.V, F.VG, p, i, j, k);
+    }
+    __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x) {
         int i, j, k;
         cell_of(c, n, D, i, j, k);
-        const int I0 = b.ijk[0] * n + i, I1 = b.ijk[1] * n + j, I2 = b.ijk[2] * n + k;
-        const int c0 = b.poff[0] + i / 2, c1 = b.poff[1] + j / 2, c2 = D == 3 ? b.poff[2] + k / 2 : 0;
-        const T v0 = load<T, D>(F.X, F.XG, p, c0, c1, c2) - load<T, D>(F.V, F.VG, p, c0, c1, c2);
-        const int sx = (I0 & 1) ? 1 : -1, sy = (I1 & 1) ? 1 : -1, sz = (I2 & 1) ? 1 : -1;
-        T nbs = load<T, D>(F.X, F.XG, p, c0 + sx, c1, c2) - load<T, D>(F.V, F.VG, p, c0 + sx, c1, c2);
-        nbs += load<T, D>(F.X, F.XG, p, c0, c1 + sy, c2) - load<T, D>(F.V, F.VG, p, c0, c1 + sy, c2);
-        if (D == 3) nbs += load<T, D>(F.X, F.XG, p, c0, c1, c2 + sz) - load<T, D>(F.V, F.VG, p, c0, c1, c2 + sz);
-        const T val = D == 2 ? ((T)2 * v0 + nbs) / (T)4 : (v0 + nbs) / (T)4;
-        const T xn = F.X[b.cell_off + c] + val;
+        // blocks start at even cells: the local parity is the global one
+        const T *d = box + (D == 3 ? (k / 2 + 1) * B * B : 0) + (j / 2 + 1) * B + i / 2 + 1;
+        T nbs = d[(i & 1) ? 1 : -1];
+        nbs += d[(j & 1) ? B : -B];
+        if (D == 3) nbs += d[(k & 1) ? B * B : -B * B];
+        const T xn = F.X[b.cell_off + c] + (D == 2 ? (T)2 * d[0] + nbs : d[0] + nbs) * (T)0.25;
         F.X[b.cell_off + c] = xn;
         xs[c] = xn;
     }
@@ -1624,6 +1656,7 @@ __global__ void __launch_bounds__(128) k_prolong_rows(KParams P, int first, int 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ int s_abort;
+    __shared__ T dbox[sizeof(T) == 8 ? 216 : 1];  // FP64: x^H - x^H_old on the octant and its face halo
     T *stage0 = reinterpret_cast<T *>(smem_raw);
     const int tid = threadIdx.x;
     constexpr int ISSUER = 127;  // stage copies and stores
@@ -1710,8 +1743,39 @@ __global__ void __launch_bounds__(128) k_prolong_rows(KParams P, int first, int 
         // the cells' y and z sides, parent ghosts where these leave the parent
         T v[4];
         const int cfm = cf_faces(b, 3);
+        if constexpr (sizeof(T) == 8) {
+            // FP64: each difference x^H - x^H_old once, on the octant and its
+            // face halo (a thread forming its own ten took 10 of 30 FP64
+            // instructions a half row, and GB300's FP64 unit bounds this form)
+            for (int q = tid; q < 216; q += 128) {
+                const int a = q % 6, c = (q / 6) % 6, e = q / 36;
+                if ((a == 0 || a == 5) + (c == 0 || c == 5) + (e == 0 || e == 5) > 1) continue;  // never read
+                const int i = b.poff[0] + a - 1, jj = b.poff[1] + c - 1, kk = b.poff[2] + e - 1;
+                int at, g = 1;  // in the ghosts, else in the block
+                if (i < 0) at = jj + 8 * kk;
+                else if (i >= n) at = FC + jj + 8 * kk;
+                else if (jj < 0) at = 2 * FC + i + 8 * kk;
+                else if (jj >= n) at = 3 * FC + i + 8 * kk;
+                else if (kk < 0) at = 4 * FC + i + 8 * jj;
+                else if (kk >= n) at = 5 * FC + i + 8 * jj;
+                else { at = i + 8 * (jj + 8 * kk); g = 0; }
+                dbox[q] = (g ? pg : px)[at] - (g ? pvg : pv)[at];
+            }
+            __syncthreads();
+        }
         {
             const int p0 = b.poff[0] + 2 * h, pj = b.poff[1] + (j >> 1), pk = b.poff[2] + (k >> 1);
+            T *xr = xs + 8 * r + 4 * h;
+#pragma unroll
+            for (int q = 0; q < 4; q += VW) vscatter(v + q, *reinterpret_cast<const V *>(xr + q));
+            if constexpr (sizeof(T) == 8) {
+                const T *d = dbox + (k / 2 + 1) * 36 + (j / 2 + 1) * 6 + 2 * h + 1;
+                const T s0 = d[0] + d[6 * sy] + d[36 * sz], s1 = d[1] + d[1 + 6 * sy] + d[1 + 36 * sz];
+                v[0] = fma((T)0.25, s0 + d[-1], v[0]);
+                v[1] = fma((T)0.25, s0 + d[1], v[1]);
+                v[2] = fma((T)0.25, s1 + d[0], v[2]);
+                v[3] = fma((T)0.25, s1 + d[2], v[3]);
+            } else {
             auto dx = [&](const T *x, const T *o, int idx) { return x[idx] - o[idx]; };
             const int row = 8 * (pj + 8 * pk);
             const T xm = p0 > 0 ? dx(px, pv, row + p0 - 1) : dx(pg, pvg, pj + 8 * pk);
@@ -1726,15 +1790,13 @@ __global__ void __launch_bounds__(128) k_prolong_rows(KParams P, int first, int 
             const T z1 = rz >= 0 ? dx(px, pv, rz + p0 + 1) : dx(pg, pvg, gz + p0 + 1);
             const T c0[4] = {x0, x0, x1, x1}, cx[4] = {xm, x1, x0, xp};
             const T cy[4] = {y0, y0, y1, y1}, cz[4] = {z0, z0, z1, z1};
-            T *xr = xs + 8 * r + 4 * h;
-#pragma unroll
-            for (int q = 0; q < 4; q += VW) vscatter(v + q, *reinterpret_cast<const V *>(xr + q));
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 T nbs = cx[q];
                 nbs += cy[q];
                 nbs += cz[q];
                 v[q] = v[q] + (c0[q] + nbs) / (T)4;
+            }
             }
             // the corrected cells go straight to global memory (16-byte
             // stores, a warp's rows contiguous); the stage keeps them only
@@ -2041,6 +2103,44 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
             if (kk < 0 || kk >= n) return gi[(s ? 5 : 4) * FC + i + n * j];
             return xi[cidx<D>(n, i, j, kk)];
         };
+        const int pn = p.n;
+        bool done = false;
+        if constexpr (sizeof(T) == 8) {
+            // FP64, constant coefficient: the Laplacians of the 2^D children
+            // of a parent cell share their inner faces, whose fluxes cancel.
+            // What is left is sum_d w_d (outer neighbours in d - children):
+            // 5 instead of 16 FP64 instructions a child in 3D, and no pass
+            // over the child residuals (128^3 Jacobi solve: 44 -> 20 us a launch).
+            if (!var && !cyl) {
+                done = true;
+                const T wsum = ih0 + ih1 + (D == 3 ? ih2 : (T)0) + kp_helm<T>(P), inv = (T)(1.0 / (1 << D));
+                for (int c = tid; c < M; c += nth) {
+                    const int ci = c % m, cj = (c / m) % m, ck = D == 3 ? c / (m * m) : 0;
+                    T sx = 0, sf = 0, ox = 0, oy = 0, oz = 0;
+#pragma unroll
+                    for (int g = 0; g < (D == 3 ? 2 : 1); g++)
+#pragma unroll
+                        for (int e = 0; e < 2; e++) {  // the row of two children at j + e, k + g
+                            const int i = 2 * ci, j = 2 * cj + e, k = D == 3 ? 2 * ck + g : 0, fc = cidx<D>(n, i, j, k);
+                            sx += xs[fc] + xs[fc + 1];
+                            sf += fs[fc] + fs[fc + 1];
+                            ox += nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i + 1, j, k, 0, 1);
+                            oy += nbv(xs, gs, i, j, k, 1, e) + nbv(xs, gs, i + 1, j, k, 1, e);
+                            if (D == 3) oz += nbv(xs, gs, i, j, k, 2, g) + nbv(xs, gs, i + 1, j, k, 2, g);
+                        }
+                    T r = fma(wsum, sx, sf);
+                    r = fma(-ih0, ox, r);
+                    r = fma(-ih1, oy, r);
+                    if (D == 3) r = fma(-ih2, oz, r);
+                    const T xv = sx * inv;
+                    const int pc = cidx<D>(pn, b.poff[0] + ci, b.poff[1] + cj, b.poff[2] + ck);
+                    F.X[p.cell_off + pc] = xv;
+                    F.F[p.cell_off + pc] = r * inv;
+                    rs[c] = xv;
+                }
+            }
+        }
+        if (!done) {
         // child residuals (same arithmetic as the stencil helper)
         for (int c = tid; c < C; c += nth) {
             const int i = c % n, j = (c / n) % n, k = D == 3 ? c / (n * n) : 0;
@@ -2092,6 +2192,7 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
                 sx += xs[cidx<D>(n, 2 * ci + (ch & 1), 2 * cj + ((ch >> 1) & 1), D == 3 ? 2 * ck + ((ch >> 2) & 1) : 0)];
             rs[c] = sx * (T)(1.0 / (1 << D));
         }
+        }
         __syncthreads();
         const int Fm = face_of<D>(m);
         auto val = [&](I3 q) { return rs[cidx<D>(m, q.x - b.poff[0], q.y - b.poff[1], q.z - b.poff[2])]; };
@@ -2102,44 +2203,6 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
             I3 ii = face_cell<D>(m, face, v, false);
             ii.x += b.poff[0];
             ii.y += b.poff[1];
-        const int pn = p.n;
-        bool done = false;
-        if constexpr (sizeof(T) == 8) {
-            // FP64, constant coefficient: the Laplacians of the 2^D children
-            // of a parent cell share their inner faces, whose fluxes cancel.
-            // What is left is sum_d w_d (outer neighbours in d - children):
-            // 5 instead of 16 FP64 instructions a child in 3D, and no pass
-            // over the child residuals (128^3 Jacobi solve: 44 -> 20 us a launch).
-            if (!var && !cyl) {
-                done = true;
-                const T wsum = ih0 + ih1 + (D == 3 ? ih2 : (T)0) + kp_helm<T>(P), inv = (T)(1.0 / (1 << D));
-                for (int c = tid; c < M; c += nth) {
-                    const int ci = c % m, cj = (c / m) % m, ck = D == 3 ? c / (m * m) : 0;
-                    T sx = 0, sf = 0, ox = 0, oy = 0, oz = 0;
-#pragma unroll
-                    for (int g = 0; g < (D == 3 ? 2 : 1); g++)
-#pragma unroll
-                        for (int e = 0; e < 2; e++) {  // the row of two children at j + e, k + g
-                            const int i = 2 * ci, j = 2 * cj + e, k = D == 3 ? 2 * ck + g : 0, fc = cidx<D>(n, i, j, k);
-                            sx += xs[fc] + xs[fc + 1];
-                            sf += fs[fc] + fs[fc + 1];
-                            ox += nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i + 1, j, k, 0, 1);
-                            oy += nbv(xs, gs, i, j, k, 1, e) + nbv(xs, gs, i + 1, j, k, 1, e);
-                            if (D == 3) oz += nbv(xs, gs, i, j, k, 2, g) + nbv(xs, gs, i + 1, j, k, 2, g);
-                        }
-                    T r = fma(wsum, sx, sf);
-                    r = fma(-ih0, ox, r);
-                    r = fma(-ih1, oy, r);
-                    if (D == 3) r = fma(-ih2, oz, r);
-                    const T xv = sx * inv;
-                    const int pc = cidx<D>(pn, b.poff[0] + ci, b.poff[1] + cj, b.poff[2] + ck);
-                    F.X[p.cell_off + pc] = xv;
-                    F.F[p.cell_off + pc] = r * inv;
-                    rs[c] = xv;
-                }
-            }
-        }
-        if (!done) {
             ii.z += D == 3 ? b.poff[2] : 0;
             put(ii, d, s ? pn - 1 : 0);
             int u;
@@ -2192,7 +2255,6 @@ __global__ void __launch_bounds__(128) k_restrict_rows(KParams P, int first, int
         }
     };
     auto parent = [&](int g, Src &r) {
-        }
         if (g < nblocks) r.plev = P.B[r.par].lev;
     };
     auto issue = [&](int it, int g, const Src &r) {  // thread ISSUER only
@@ -3770,9 +3832,29 @@ __global__ void __launch_bounds__(256) k_jacobi_flat(KParams P, int first, int n
         const int c = (int)(idx % C);
         int i, j, k;
         cell_of(c, n, D, i, j, k);
-        T lap, num, den, xc;
-        stencil<T, T, D>(P, L, b, F.X, F.XG, F.E, F.EG, i, j, k, lap, num, den, xc);
-        const T xgs = qdiv<T>(num - F.F[b.cell_off + c], den + kp_helm<T>(P));
+        T xc, xgs;
+        if (!F.E && P.geom == MG_CART) {  // one weight per dimension, the row's diagonal divided out
+            auto x = [&](int a, int e, int g) { return load<T, D>(F.X, F.XG, b, a, e, g); };
+            xc = F.X[b.cell_off + c];
+            xgs = -F.F[b.cell_off + c] * lv_idiag<T>(L);
+            xgs = lv_wd<T>(L, 0) * (x(i - 1, j, k) + x(i + 1, j, k)) + xgs;
+            xgs = lv_wd<T>(L, 1) * (x(i, j - 1, k) + x(i, j + 1, k)) + xgs;
+            if (D == 3) xgs = lv_wd<T>(L, 2) * (x(i, j, k - 1) + x(i, j, k + 1)) + xgs;
+        } else if (F.W) {  // FP64: coefficients and 1 / diagonal precomputed
+            const T *ws = F.W + b.cell_off * wstride(D) + c;
+            xc = F.X[b.cell_off + c];
+            T num = -F.F[b.cell_off + c];
+#pragma unroll
+            for (int f = 0; f < 2 * D; f++) {
+                const int d = f >> 1, o = (f & 1) ? 1 : -1;
+                num += ws[f * C] * load<T, D>(F.X, F.XG, b, i + (d == 0 ? o : 0), j + (d == 1 ? o : 0), k + (d == 2 ? o : 0));
+            }
+            xgs = num * ws[(2 * D + 1) * C];
+        } else {
+            T lap, num, den;
+            stencil<T, T, D>(P, L, b, F.X, F.XG, F.E, F.EG, i, j, k, lap, num, den, xc);
+            xgs = qdiv<T>(num - F.F[b.cell_off + c], den + kp_helm<T>(P));
+        }
         F.J[b.cell_off + c] = xc + omega * (xgs - xc);
     }
 }
@@ -4515,7 +4597,7 @@ template <class T, int D> struct Launch {
             ghost(t, P, l, F.X, F.XG, 0);
             return;
         }
-        const size_t sm = sizeof(T) * cells_of<D>(L.n);
+        const size_t sm = sizeof(T) * (cells_of<D>(L.n) + cells_of<D>(L.n / 2 + 2));
         set_smem(k_prolong_push<T, D>, sm);
         launch_k(k_prolong_push<T, D>, L.nb, threads_for(cells_of<D>(L.n)), sm, t->stream, P, L.first, F);
     }

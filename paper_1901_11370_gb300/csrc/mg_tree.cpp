@@ -492,6 +492,8 @@ static int upload_bc(mg_tree *t) {
             for (int e = 0; e < t->dim; e++) sw += d.inv_h2[e];
             d.diag = 2.0 * sw + t->helm;
             d.inv_diag = 1.0 / d.diag;
+            for (int e = 0; e < 3; e++) d.wd[e] = d.inv_h2[e] / d.diag;
+            d.pad = 0.0;
             d.vol = L.h[0] * L.h[1] * (t->dim == 3 ? L.h[2] : 1.0);
             for (int e = 0; e < 3; e++) d.inv_h2f[e] = (float)d.inv_h2[e];
             d.inv_diagf = (float)d.inv_diag;
