@@ -295,6 +295,10 @@ struct mg_tree {
     };
     std::map<std::string, Graph> graphs;
     cudaStream_t cap_stream = nullptr;
+    bool capturing = false;            // inside run_graph's capture
+    std::vector<cudaStream_t> aux;     // side streams of a capture's parallel branches (at most kAux)
+    std::vector<cudaEvent_t> ev_join;
+    cudaEvent_t ev_fork = nullptr;
     bool use_graphs = true;
     std::vector<int> sweep_choice[2];  // autotuned sweep variant per level (FP64, FP32); -1 default
     // the tail kernel (mg_kernels.cu): cell bound of the groups it runs
@@ -331,6 +335,7 @@ template <class T> void refresh_eps(mg_tree *t, Fields<T> &F);
 template <class T> void tune_sweeps(mg_tree *t, Fields<T> &F);
 int sweep_variant(mg_tree *t, int prec, int level);
 constexpr int kNumSweepVariants = 11;
+constexpr int kAux = 12;  // parallel branches of a captured step beside the stream itself
 constexpr int kCoarseRows = 8;  // rows of one tree per CTA of the coarse apply
 constexpr int kBtResidCells = 256;  // cells per CTA of the block-form coarsest residual
 bool sweep_variant_ok(mg_tree *t, int prec, int level, int variant);

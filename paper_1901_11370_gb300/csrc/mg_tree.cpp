@@ -1027,7 +1027,9 @@ template <class Fn> static int run_graph(mg_tree *t, const std::string &key, Fn 
         CK(cudaStreamSynchronize(user));
         t->stream = t->cap_stream;
         cudaError_t e = cudaStreamBeginCapture(t->cap_stream, cudaStreamCaptureModeRelaxed);
+        t->capturing = e == cudaSuccess;
         if (e == cudaSuccess) enqueue();
+        t->capturing = false;
         const std::string le = take_launch_error();  // a launch refused during capture is missing from the graph
         cudaGraph_t g = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(t->cap_stream, &g);
@@ -1729,6 +1731,9 @@ extern "C" int mg_tree_destroy(mg_tree *t) {
         cudaFreeHost(t->h_tree3);
         drop_graphs(t);
         if (t->cap_stream) cudaStreamDestroy(t->cap_stream);
+        for (cudaStream_t s : t->aux) cudaStreamDestroy(s);
+        for (cudaEvent_t e : t->ev_join) cudaEventDestroy(e);
+        if (t->ev_fork) cudaEventDestroy(t->ev_fork);
     }
     delete t;
     return MG_OK;
