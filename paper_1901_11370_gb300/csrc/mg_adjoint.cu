@@ -439,10 +439,10 @@ template <int D> struct Adj {
             launch_k(k_restrict_T<D>, L.nb, threads_of(cells_of<D>(L.n)), 0, t->stream, P, L.first, t->d_at);
         }
     }
-    // leaf-vector op over all leaf blocks; with a reduction, the two sums
-    // arrive on the host (synchronises the stream)
+    // leaf-vector op over all leaf blocks, enqueued only; with a reduction,
+    // the two sums land in the pinned h_red (wait reads them)
     static void vec(mg_tree *t, const KParams &P, int op, const double *la, const double *lb, double *lo,
-                    const double *ca, double *co, double scal, double *sums) {
+                    const double *ca, double *co, double scal, bool reduce) {
         long long leaf_base = 0;
         int slot = 0;
         for (const LevelHost &L : t->lev) {
@@ -454,9 +454,11 @@ template <int D> struct Adj {
             slot += nleaf;
             leaf_base += (long long)nleaf * cells_of<D>(L.n);
         }
-        if (!sums) return;
+        if (!reduce) return;
         ++t->launches;
         launch_k(k_sum_partials, 1, kSumThreads, 0, t->stream, (const double *)t->d_partials, slot, t->h_red);  // pinned
+    }
+    static void wait(mg_tree *t, double *sums) {
         cudaStreamSynchronize(t->stream);
         sums[0] = t->h_red[0];
         sums[1] = t->h_red[1];
@@ -498,47 +500,66 @@ void eps_grad_transpose(mg_tree *t, const double *lam, double *out) {
 // until the volume-weighted norm of W^-1 (g - A^T lambda) is at most rel_tol
 // times that of W^-1 g, or max_it iterations.  Singular problems: g is made
 // compatible (sum g = 0) and lambda returned as lambda - W sum(lambda) / sum W.
+// lambda stays in the tree's own buffer (t->d_lam), so that the start and an
+// iteration are captured graphs whose pointers do not change between calls:
+// an iteration is 30 to 60 launches, which cost more to enqueue than a mesh
+// of 64^3 cells to run.  key: the graph-key suffix of the cycle parameters.
 template <int D>
-static int adjoint_dc_d(mg_tree *t, const double *g, double *lam, int nd, int nu, double rel_tol, int max_it,
-                        int *it_out, double *rel_out, bool fp32) {
+static int adjoint_dc_d(mg_tree *t, const double *g, int nd, int nu, double rel_tol, int max_it, int *it_out,
+                        double *rel_out, bool fp32, const std::string &key) {
     const KParams P = kparams(t, 1);
-    double s[2];
+    double s[2], *lam = t->d_lam;
+    int rc;
     cudaMemcpyAsync(t->d_gh, g, sizeof(double) * (size_t)t->nleaf_cells, cudaMemcpyDeviceToDevice, t->stream);
     if (t->singular) {
-        Adj<D>::vec(t, P, V_SUM, t->d_gh, nullptr, nullptr, nullptr, nullptr, 0.0, s);
-        Adj<D>::vec(t, P, V_PROJ, t->d_gh, nullptr, t->d_gh, nullptr, nullptr, s[1] > 0 ? s[0] / s[1] : 0.0, nullptr);
+        Adj<D>::vec(t, P, V_SUM, t->d_gh, nullptr, nullptr, nullptr, nullptr, 0.0, true);
+        Adj<D>::wait(t, s);
+        Adj<D>::vec(t, P, V_PROJ, t->d_gh, nullptr, t->d_gh, nullptr, nullptr, s[1] > 0 ? s[0] / s[1] : 0.0, false);
     }
-    Adj<D>::vec(t, P, V_INIT, t->d_gh, nullptr, nullptr, nullptr, t->adj.F, 0.0, s);
+    Adj<D>::vec(t, P, V_INIT, t->d_gh, nullptr, nullptr, nullptr, t->adj.F, 0.0, true);
+    Adj<D>::wait(t, s);
     const double r0 = s[1] > 0 ? std::sqrt(s[0] / s[1]) : 0.0;
-    cudaMemsetAsync(t->adj.X, 0, sizeof(double) * (size_t)t->ncells, t->stream);
-    cudaMemsetAsync(t->adj.XG, 0, sizeof(double) * (size_t)t->nghost, t->stream);
-    fmg<double>(t, t->adj, nd, nu, 1);
-    Adj<D>::vec(t, P, V_SET, nullptr, nullptr, lam, t->adj.X, nullptr, 0.0, nullptr);
+    auto residual = [&] {  // W^-1 (g - A^T lambda) into adj.F, its norm
+        apply_T_d<D>(t, lam, t->d_lv);
+        Adj<D>::vec(t, P, V_RESID, t->d_gh, t->d_lv, nullptr, nullptr, t->adj.F, 0.0, true);
+    };
+    rc = run_graph_fn(t, "adj-start" + key, [&] {
+        cudaMemsetAsync(t->adj.X, 0, sizeof(double) * (size_t)t->ncells, t->stream);
+        cudaMemsetAsync(t->adj.XG, 0, sizeof(double) * (size_t)t->nghost, t->stream);
+        fmg<double>(t, t->adj, nd, nu, 1);
+        Adj<D>::vec(t, P, V_SET, nullptr, nullptr, lam, t->adj.X, nullptr, 0.0, false);
+        residual();
+    });
+    if (rc) return rc;
     const int top = (int)t->groups.size() - 1;
     int it = 0;
     double rel = 0.0;
     for (;;) {
-        apply_T_d<D>(t, lam, t->d_lv);
-        Adj<D>::vec(t, P, V_RESID, t->d_gh, t->d_lv, nullptr, nullptr, t->adj.F, 0.0, s);
+        Adj<D>::wait(t, s);
         rel = r0 > 0 ? std::sqrt(s[0] / s[1]) / r0 : 0.0;
         if (it >= max_it || rel <= rel_tol || !std::isfinite(rel)) break;
-        if (fp32) {  // the FP32 V-cycle on the residual's FP32 copy, as in the forward solve's defect correction
-            narrow_f32(t, t->adj.F, t->f32.F, t->ncells);
-            cudaMemsetAsync(t->f32.X, 0, sizeof(float) * (size_t)t->ncells, t->stream);
-            cudaMemsetAsync(t->f32.XG, 0, sizeof(float) * (size_t)t->nghost, t->stream);
-            vcycle<float>(t, t->f32, top, nd, nu, 1);
-            widen_f64(t, t->f32.X, t->adj.X, t->ncells);
-        } else {
-            cudaMemsetAsync(t->adj.X, 0, sizeof(double) * (size_t)t->ncells, t->stream);
-            cudaMemsetAsync(t->adj.XG, 0, sizeof(double) * (size_t)t->nghost, t->stream);
-            vcycle<double>(t, t->adj, top, nd, nu, 1);
-        }
-        Adj<D>::vec(t, P, V_ADD, nullptr, nullptr, lam, t->adj.X, nullptr, 0.0, nullptr);
+        rc = run_graph_fn(t, (fp32 ? "adj-it32" : "adj-it64") + key, [&] {
+            if (fp32) {  // the FP32 V-cycle on the residual's FP32 copy, as in the forward solve's defect correction
+                narrow_f32(t, t->adj.F, t->f32.F, t->ncells);
+                cudaMemsetAsync(t->f32.X, 0, sizeof(float) * (size_t)t->ncells, t->stream);
+                cudaMemsetAsync(t->f32.XG, 0, sizeof(float) * (size_t)t->nghost, t->stream);
+                vcycle<float>(t, t->f32, top, nd, nu, 1);
+                widen_f64(t, t->f32.X, t->adj.X, t->ncells);
+            } else {
+                cudaMemsetAsync(t->adj.X, 0, sizeof(double) * (size_t)t->ncells, t->stream);
+                cudaMemsetAsync(t->adj.XG, 0, sizeof(double) * (size_t)t->nghost, t->stream);
+                vcycle<double>(t, t->adj, top, nd, nu, 1);
+            }
+            Adj<D>::vec(t, P, V_ADD, nullptr, nullptr, lam, t->adj.X, nullptr, 0.0, false);
+            residual();
+        });
+        if (rc) return rc;
         it++;
     }
     if (t->singular) {
-        Adj<D>::vec(t, P, V_SUM, lam, nullptr, nullptr, nullptr, nullptr, 0.0, s);
-        Adj<D>::vec(t, P, V_PROJ, lam, nullptr, lam, nullptr, nullptr, s[1] > 0 ? s[0] / s[1] : 0.0, nullptr);
+        Adj<D>::vec(t, P, V_SUM, lam, nullptr, nullptr, nullptr, nullptr, 0.0, true);
+        Adj<D>::wait(t, s);
+        Adj<D>::vec(t, P, V_PROJ, lam, nullptr, lam, nullptr, nullptr, s[1] > 0 ? s[0] / s[1] : 0.0, false);
     }
     if (it_out) *it_out = it;
     if (rel_out) *rel_out = rel;
@@ -546,9 +567,12 @@ static int adjoint_dc_d(mg_tree *t, const double *g, double *lam, int nd, int nu
 }
 
 int adjoint_dc(mg_tree *t, const double *g, double *lam, int nd, int nu, double rel_tol, int max_it, int *it_out,
-               double *rel_out, bool fp32) {
-    return t->dim == 2 ? adjoint_dc_d<2>(t, g, lam, nd, nu, rel_tol, max_it, it_out, rel_out, fp32)
-                       : adjoint_dc_d<3>(t, g, lam, nd, nu, rel_tol, max_it, it_out, rel_out, fp32);
+               double *rel_out, const std::string &key, bool fp32) {
+    const int rc = t->dim == 2 ? adjoint_dc_d<2>(t, g, nd, nu, rel_tol, max_it, it_out, rel_out, fp32, key)
+                               : adjoint_dc_d<3>(t, g, nd, nu, rel_tol, max_it, it_out, rel_out, fp32, key);
+    if (rc) return rc;
+    cudaMemcpyAsync(lam, t->d_lam, sizeof(double) * (size_t)t->nleaf_cells, cudaMemcpyDeviceToDevice, t->stream);
+    return check_cuda("adjoint");
 }
 
 // Vector-Jacobian product of the cleaning map B -> B - G phi, phi the
@@ -557,7 +581,7 @@ int adjoint_dc(mg_tree *t, const double *g, double *lam, int nd, int nu, double 
 // singular problem applied inside adjoint_dc.
 template <int D>
 static int clean_adjoint_d(mg_tree *t, const double *gBn, double *gB, int nd, int nu, double rel_tol, int max_it,
-                           int *it_out, double *rel_out, bool fp32) {
+                           int *it_out, double *rel_out, bool fp32, const std::string &key) {
     const KParams P = kparams(t, 1);
     const long long nl = t->nleaf_cells;
     // u = G^T gBn into gB's first component (free until the end)
@@ -565,21 +589,21 @@ static int clean_adjoint_d(mg_tree *t, const double *gBn, double *gB, int nd, in
     Adj<D>::refresh_T(t, P, G_PHI);
     double *u = gB;
     cells_to_leaf(t, t->d_at, u);
-    int rc = adjoint_dc_d<D>(t, u, t->d_lam, nd, nu, rel_tol, max_it, it_out, rel_out, fp32);
+    int rc = adjoint_dc_d<D>(t, u, nd, nu, rel_tol, max_it, it_out, rel_out, fp32, key);
     if (rc) return rc;
     for (int d = 0; d < D; d++) {
         Adj<D>::stencil(t, P, T_DIV, d, t->d_lam, nullptr, nullptr, nullptr, nullptr);
         Adj<D>::refresh_T(t, P, G_VEC);
         cells_to_leaf(t, t->d_at, t->d_lv);
-        Adj<D>::vec(t, P, V_SUB, gBn + d * nl, t->d_lv, gB + d * nl, nullptr, nullptr, 0.0, nullptr);
+        Adj<D>::vec(t, P, V_SUB, gBn + d * nl, t->d_lv, gB + d * nl, nullptr, nullptr, 0.0, false);
     }
     return check_cuda("clean adjoint");
 }
 
 int clean_adjoint(mg_tree *t, const double *gBn, double *gB, int nd, int nu, double rel_tol, int max_it, int *it_out,
-                  double *rel_out, bool fp32) {
-    return t->dim == 2 ? clean_adjoint_d<2>(t, gBn, gB, nd, nu, rel_tol, max_it, it_out, rel_out, fp32)
-                       : clean_adjoint_d<3>(t, gBn, gB, nd, nu, rel_tol, max_it, it_out, rel_out, fp32);
+                  double *rel_out, const std::string &key, bool fp32) {
+    return t->dim == 2 ? clean_adjoint_d<2>(t, gBn, gB, nd, nu, rel_tol, max_it, it_out, rel_out, fp32, key)
+                       : clean_adjoint_d<3>(t, gBn, gB, nd, nu, rel_tol, max_it, it_out, rel_out, fp32, key);
 }
 
 }  // namespace mg

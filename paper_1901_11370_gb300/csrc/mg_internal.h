@@ -2,6 +2,7 @@
 // CUDA kernels and cycle driver (mg_kernels.cu).  Not part of the public ABI.
 #pragma once
 #include <cstdint>
+#include <functional>
 #include <map>
 #include <string>
 #include <vector>
@@ -388,9 +389,11 @@ void eps_grad_transpose(mg_tree *t, const double *lam, double *out);
 // fp32: FP32 V-cycles (the tree's FP32 set, allocated) as the approximate
 // inverse inside the FP64 defect correction, else FP64 V-cycles
 int adjoint_dc(mg_tree *t, const double *g, double *lam, int nd, int nu, double rel_tol, int max_it, int *it_out,
-               double *rel_out, bool fp32 = false);
+               double *rel_out, const std::string &key, bool fp32 = false);
 int clean_adjoint(mg_tree *t, const double *gBn, double *gB, int nd, int nu, double rel_tol, int max_it,
-                  int *it_out, double *rel_out, bool fp32 = false);
+                  int *it_out, double *rel_out, const std::string &key, bool fp32 = false);
+// enqueue() as a graph captured once per key and replayed (mg_tree.cpp)
+int run_graph_fn(mg_tree *t, const std::string &key, const std::function<void()> &enqueue);
 }  // namespace mg
 
 void mg_set_error(const std::string &msg);

@@ -1058,6 +1058,10 @@ template <class Fn> static int run_graph(mg_tree *t, const std::string &key, Fn 
     return MG_OK;
 }
 
+int mg::run_graph_fn(mg_tree *t, const std::string &key, const std::function<void()> &enqueue) {
+    return run_graph(t, key, enqueue);
+}
+
 extern "C" int mg_set_bc_plane(mg_tree *t, int face, int level, const double *vals) {
     if (!t || !vals) return fail(MG_ERR_ARG, "null argument");
     int rc = build(t);
@@ -1389,7 +1393,7 @@ static bool has_refinement_faces(const mg_tree *t) {
     return false;
 }
 
-static int adjoint_setup(mg_tree *t, const mg_params *p, mg_params *q) {
+static int adjoint_setup(mg_tree *t, const mg_params *p, mg_params *q, std::string *key) {
     if (t->is_batch) return fail(MG_ERR_UNSUPPORTED, "the adjoint works on one tree, not a batch");
     // a singular problem's compatibility condition is sum V f = 0 only where
     // fluxes are conserved; with variable eps at refinement faces they are
@@ -1398,7 +1402,7 @@ static int adjoint_setup(mg_tree *t, const mg_params *p, mg_params *q) {
         return fail(MG_ERR_UNSUPPORTED, "adjoint of a problem without Dirichlet faces needs constant eps on a "
                                         "mesh with refinement faces");
     int rc;
-    if ((rc = use_params(t, p, q, nullptr))) return rc;
+    if ((rc = use_params(t, p, q, key))) return rc;
     if (q->precision == MG_FP32_DC && (rc = ensure_f32(t))) return rc;
     if ((rc = alloc_fields(t, t->adj, false))) return rc;
     t->adj.E = t->f64.E;
@@ -1418,8 +1422,9 @@ static int adjoint_run(mg_tree *t, const double *g, double *dLdf, double *dLdeps
     mg_params q;
     int rc, it = 0;
     double rel = 0.0;
-    if ((rc = adjoint_setup(t, p, &q))) return rc;
-    if ((rc = adjoint_dc(t, g, dLdf, q.n_down, q.n_up, rel_tol, max_cycles, &it, &rel, q.precision == MG_FP32_DC)))
+    std::string key;
+    if ((rc = adjoint_setup(t, p, &q, &key))) return rc;
+    if ((rc = adjoint_dc(t, g, dLdf, q.n_down, q.n_up, rel_tol, max_cycles, &it, &rel, key, q.precision == MG_FP32_DC)))
         return rc;
     if (dLdeps) eps_grad_transpose(t, dLdf, dLdeps);
     if ((rc = check_cuda("adjoint")) || (rc = check_status(t))) return rc;
@@ -1461,8 +1466,9 @@ extern "C" int mg_clean_adjoint(mg_tree *t, const double *gBnew, double *gB, con
     mg_params q;
     int rc, it = 0;
     double rel = 0.0;
-    if ((rc = adjoint_setup(t, p, &q))) return rc;
-    if ((rc = clean_adjoint(t, gBnew, gB, q.n_down, q.n_up, rel_tol, max_cycles, &it, &rel,
+    std::string key;
+    if ((rc = adjoint_setup(t, p, &q, &key))) return rc;
+    if ((rc = clean_adjoint(t, gBnew, gB, q.n_down, q.n_up, rel_tol, max_cycles, &it, &rel, key,
                             q.precision == MG_FP32_DC)))
         return rc;
     if ((rc = check_status(t))) return rc;
