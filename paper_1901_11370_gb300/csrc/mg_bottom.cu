@@ -635,8 +635,8 @@ template <class T, int D, bool VAR> struct Bottom {
     //   dx = Q_a Q_b G Q_b^T Q_a^T r,  G(ka, kb) = Q_p diag(1 / lambda) Q_p^T.
     // A + B + P FMAs per cell and direction instead of a row of the dense
     // inverse per cell (GB300 completes one FP64 instruction per SM in 16
-    // cycles, and the inverse is 2 to 8 MB): 7.7 us against 26 for 36 x 27
-    // cells, 13 against 14 for 8^3.  Forward along a and b the CTA
+    // cycles, and the inverse is 2 to 8 MB); the line between the two is drawn
+    // where the layout is made.  Forward along a and b the CTA
     // works on its own planes of p and its own b (as kb), then every CTA
     // gathers the transform and solves its planes.
     __device__ void coarse_fd() const {
@@ -973,7 +973,11 @@ template <class T> static size_t bot_layout(const mg_tree *t, BotPlan &B, int to
     B.mb = (B.n0[1] + B.PB - 1) / B.PB;
     B.mp = (B.n0[2] + B.PP - 1) / B.PP;
     const long long tab = (long long)B.n0[0] * B.n0[0] + (D == 3 ? (long long)B.n0[1] * B.n0[1] : 0);
-    B.fd = !t->var_eps && tab <= 2600;
+    // by eigenvectors from 400 cells on: 7.7 against 26 us for 36 x 27 cells,
+    // 13 against 14 for 8^3; below, its five dependent FP64 stages take longer
+    // than the rows of the inverse (8.0 against 6.1 for 180 cells, 5.6 against
+    // 3.7 for 8 x 8)
+    B.fd = !t->var_eps && t->nc >= 400 && tab <= 2600;
     const long long plane = (long long)B.n0[0] * (D == 3 ? B.n0[1] : 1);
     const long long scratch = B.fd ? tab + (2 * B.mp + B.n0[2]) * plane : t->ns;
     const size_t head = sizeof(double) * (size_t)(16 + scratch);
