@@ -1008,6 +1008,188 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 8 ? ((FG && STAGES == 2) 
     if (lane == 0) bulk_wait0();
 }
 
+// Quarter-row form of the sweep for 3D 16^3 blocks in FP32 (Cartesian,
+// constant or variable eps), one 512-thread CTA per SM.  What bounds
+// k_sweep_tma there is twofold: one block ahead in a double-buffered stage is
+// 60 KB in flight per SM, less than the memory's latency asks for, and its
+// per-cell index arithmetic and boundary branches (about 150 instructions a
+// cell with variable eps).  Here three stages keep two blocks in flight, and
+// a thread takes two quarter rows (4 cells, 2 of the colour): its row and
+// the four neighbour rows of x and eps come in with 16-byte loads, one face
+// ghost row in place of a row outside the block, and the face weights are
+// formed as e_n / (e_c + e_n), the factor 2 e_c of all six taken out of the
+// sums.  Ghost pushes as in k_sweep_tma.
+constexpr int kRows16Stages = 3;
+template <bool VAR>
+__global__ void __launch_bounds__(512, 1) k_sweep_rows16(KParams P, int first, int nblocks, Fields<float> F, int colour) {
+    pdl_entry();
+    using T = float;
+    constexpr int n = 16, C = 4096, FC = 256, GH = 1536, TPB = 512, GPT = GH / TPB, ST = kRows16Stages;
+    constexpr int DESC = (int)((sizeof(BlockDesc) + sizeof(LevelDesc)) / sizeof(T));
+    constexpr int STAGE = DESC + 2 * C + GH + (VAR ? C + GH : 0);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bars[ST];
+    __shared__ int s_abort;
+    T *stage0 = reinterpret_cast<T *>(smem_raw);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        for (int q = 0; q < ST; q++) mbar_init(&bars[q], 1);
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    __syncthreads();
+    auto issue = [&](int it, int g, long long co, long long go, int lev) {  // thread 0 only
+        T *st = stage0 + (it % ST) * STAGE;
+        uint64_t *bar = &bars[it % ST];
+        fence_async_smem();
+        mbar_expect_tx(bar, (uint32_t)(sizeof(T) * STAGE));
+        bulk_g2s(st, P.B + g, sizeof(BlockDesc), bar);
+        bulk_g2s(reinterpret_cast<char *>(st) + sizeof(BlockDesc), P.L + lev, sizeof(LevelDesc), bar);
+        bulk_g2s(st + DESC, F.X + co, sizeof(T) * C, bar);
+        bulk_g2s(st + DESC + C, F.XG + go, sizeof(T) * GH, bar);
+        bulk_g2s_f<T>(st + DESC + C + GH, F.F + co, sizeof(T) * C, bar);
+        if (VAR) {
+            bulk_g2s_f<T>(st + DESC + 2 * C + GH, F.E + co, sizeof(T) * C, bar);
+            bulk_g2s_f<T>(st + DESC + 3 * C + GH, F.EG + go, sizeof(T) * GH, bar);
+        }
+    };
+    const int stride = gridDim.x;
+    int g = blockIdx.x;
+    long long rco = 0, rgo = 0;
+    int rlev = 0;
+    auto fetch = [&](int gn) {  // the offsets of the block refilled next, one iteration ahead
+        if (gn < nblocks) {
+            rco = P.B[first + gn].cell_off;
+            rgo = P.B[first + gn].ghost_off;
+            rlev = P.B[first + gn].lev;
+        }
+    };
+    if (tid == 0) {
+        for (int q = 0; q < ST - 1; q++)
+            if (g + q * stride < nblocks) {
+                fetch(g + q * stride);
+                issue(q, first + g + q * stride, rco, rgo, rlev);
+            }
+        fetch(g + (ST - 1) * stride);
+    }
+    const T helm = kp_helm<T>(P);
+    const int q4 = 4 * (tid & 3), j = (tid >> 2) & 15, k0 = tid >> 6;  // quarter rows (q4, j, k0) and (q4, j, k0 + 8)
+    for (int it = 0; g < nblocks; it++, g += stride) {
+        if (!mbar_wait_bounded(&bars[it % ST], (it / ST) & 1, P.wait_limit)) {
+            atomicExch(P.status, 1);
+            s_abort = 1;
+        }
+        __syncthreads();
+        if (s_abort) {
+            // copies of this and the next blocks may still be landing in
+            // shared memory: let them arrive (normal bound) before the CTA exits
+            if (tid == 0)
+                for (int q = 0; q < ST - 1; q++)
+                    if (g + q * stride < nblocks)
+                        mbar_wait_bounded(&bars[(it + q) % ST], ((it + q) / ST) & 1, kWaitLimit);
+            break;
+        }
+        // every thread is past the previous block: its stage may be refilled
+        // once its bulk store has read it
+        if (tid == 0) {
+            if (g + (ST - 1) * stride < nblocks) {
+                bulk_wait_read0();
+                issue(it + ST - 1, first + g + (ST - 1) * stride, rco, rgo, rlev);
+            }
+            fetch(g + ST * stride);
+        }
+        T *st = stage0 + (it % ST) * STAGE;
+        const BlockDesc &b = *reinterpret_cast<const BlockDesc *>(st);
+        const LevelDesc &L = *reinterpret_cast<const LevelDesc *>(reinterpret_cast<const char *>(st) + sizeof(BlockDesc));
+        const T w0 = L.inv_h2f[0], w1 = L.inv_h2f[1], w2 = L.inv_h2f[2], inv_den = L.inv_diagf;
+        T *xs = st + DESC, *gs = xs + C, *fs = gs + GH, *es = fs + C, *egs = es + C;
+        const int par0 = (b.ijk[0] + b.ijk[1] + b.ijk[2]) * n;
+        // coarse-fine faces: B'/2 of this thread's ghost slots from the old
+        // interior values (see cf_half_base), before the update overwrites them
+        const int cfm = cf_faces(b, 3);
+        T bh[GPT];
+        if (cfm) {
+#pragma unroll
+            for (int r = 0; r < GPT; r++) {
+                const int t = tid + r * TPB, face = t / FC;
+                if (!((cfm >> face) & 1)) continue;
+                const int u = t - face * FC;
+                const I3 ii = face_cell<3>(n, face, u, false);
+                I3 dd = ii;
+                put(dd, face >> 1, (face & 1) ? n - 2 : 1);
+                bh[r] = cf_half_base(gs[t], xs[cidx<3>(n, ii.x, ii.y, ii.z)], xs[cidx<3>(n, dd.x, dd.y, dd.z)]);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = k0 + 8 * u, c = q4 + n * (j + n * k);
+            const bool p = ((colour + par0 + j + k) & 1) != 0;  // colour cells q4 + p and q4 + 2 + p
+            const int dn = j > 0 ? c - n : C + 2 * FC + q4 + n * k, up = j < n - 1 ? c + n : C + 3 * FC + q4 + n * k;
+            const int bk = k > 0 ? c - n * n : C + 4 * FC + q4 + n * j, fw = k < n - 1 ? c + n * n : C + 5 * FC + q4 + n * j;
+            // the x neighbour outside the quarter: right of its last cell or left of its first
+            const int ed = p ? (q4 < 12 ? c + 4 : C + FC + j + n * k) : (q4 > 0 ? c - 1 : C + j + n * k);
+            auto ld = [](const T *s) { return *reinterpret_cast<const float4 *>(s); };
+            // (gs follows xs and egs follows es, so one offset serves cells and ghosts)
+            const float4 x = ld(xs + c), xd = ld(xs + dn), xu = ld(xs + up), xb = ld(xs + bk), xf = ld(xs + fw), f = ld(fs + c);
+            const T xe = xs[ed];
+            // the two colour cells A, B and their x neighbours: l A m B for p = 0, A m B r ... shifted by one for p = 1
+            const T xl = p ? x.x : xe, xm = p ? x.z : x.y, xr = p ? xe : x.w;
+            T va, vb;
+            if (VAR) {
+                const float4 e = ld(es + c), ed4 = ld(es + dn), eu = ld(es + up), eb = ld(es + bk), ef = ld(es + fw);
+                const T ee = es[ed];
+                const T el = p ? e.x : ee, em = p ? e.z : e.y, er = p ? ee : e.w;
+                auto cell = [&](T ec, T e0, T x0, T e1, T x1, T e2, T x2, T e3, T x3, T e4, T x4, T e5, T x5, T fc) {
+                    // sum_f ih_f e_f / (e_c + e_f) x_f and its weights; 2 e_c times that is the row (Sec. 2.2)
+                    const T t0 = w0 * __fdividef(e0, ec + e0), t1 = w0 * __fdividef(e1, ec + e1);
+                    const T t2 = w1 * __fdividef(e2, ec + e2), t3 = w1 * __fdividef(e3, ec + e3);
+                    const T t4 = w2 * __fdividef(e4, ec + e4), t5 = w2 * __fdividef(e5, ec + e5);
+                    const T num = fmaf(t0, x0, t1 * x1) + fmaf(t2, x2, t3 * x3) + fmaf(t4, x4, t5 * x5);
+                    const T den = (t0 + t1) + (t2 + t3) + (t4 + t5), s = ec + ec;
+                    return __fdividef(fmaf(s, num, -fc), fmaf(s, den, helm));
+                };
+                va = cell(p ? e.y : e.x, el, xl, em, xm, p ? ed4.y : ed4.x, p ? xd.y : xd.x, p ? eu.y : eu.x, p ? xu.y : xu.x,
+                          p ? eb.y : eb.x, p ? xb.y : xb.x, p ? ef.y : ef.x, p ? xf.y : xf.x, p ? f.y : f.x);
+                vb = cell(p ? e.w : e.z, em, xm, er, xr, p ? ed4.w : ed4.z, p ? xd.w : xd.z, p ? eu.w : eu.z, p ? xu.w : xu.z,
+                          p ? eb.w : eb.z, p ? xb.w : xb.z, p ? ef.w : ef.z, p ? xf.w : xf.z, p ? f.w : f.z);
+            } else {
+                const T ya = p ? xd.y + xu.y : xd.x + xu.x, yb = p ? xd.w + xu.w : xd.z + xu.z;
+                const T za = p ? xb.y + xf.y : xb.x + xf.x, zb = p ? xb.w + xf.w : xb.z + xf.z;
+                va = (w0 * (xl + xm) + w1 * ya + w2 * za - (p ? f.y : f.x)) * inv_den;
+                vb = (w0 * (xm + xr) + w1 * yb + w2 * zb - (p ? f.w : f.z)) * inv_den;
+            }
+            // the quarter's other cells keep their values; its neighbours read only those
+            *reinterpret_cast<float4 *>(xs + c) = p ? make_float4(x.x, va, x.z, vb) : make_float4(va, x.y, vb, x.w);
+        }
+        fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+            bulk_s2g(F.X + b.cell_off, xs, sizeof(T) * C);
+            bulk_commit();
+        }
+        // ghost pushes beside updated cells (see k_sweep)
+#pragma unroll
+        for (int r = 0; r < GPT; r++) {
+            const int t = tid + r * TPB, face = t / FC, u = t - face * FC;
+            const I3 ii = face_cell<3>(n, face, u, false);
+            const bool updated = ((par0 + ii.x + ii.y + ii.z) & 1) == colour;
+            const int nb = b.nbr[face];
+            const T xi = xs[cidx<3>(n, ii.x, ii.y, ii.z)];
+            if (nb >= 0) {
+                if (updated) F.XG[b.push[face] + u] = xi;
+            } else if (nb == -1) {
+                if (updated) F.XG[b.ghost_off + t] = phys_ghost<T>(P, L, face, xi, bc_value(P, L, b, 3, face, ii));
+            } else {
+                I3 dd = ii;
+                put(dd, face >> 1, (face & 1) ? n - 2 : 1);
+                F.XG[b.ghost_off + t] = cf_from_half_base(bh[r], xi, xs[cidx<3>(n, dd.x, dd.y, dd.z)]);
+            }
+        }
+    }
+    if (tid == 0) bulk_wait0();
+}
+
 // ------------------------------------------------------- transfers ------
 // Restriction (Sec. 2.3): the parent cells under fine block b receive the
 // mean of their 2^D children; with_res also stores the mean of the child
@@ -4334,6 +4516,8 @@ template <class T, int D> struct Launch {
     //  7 / 8 / 9 row-wise warp sweep with f in registers (FP32): 8 warps x 3
     //        stages / 4 warps x 4 stages / 8 warps x 2 stages
     // 10 candidate 0 with half the threads per CTA (two colour cells each)
+    // FP32 16^3 blocks (3D): candidate 0 is k_sweep_rows16, with its three stages
+    static constexpr bool rows16() { return D == 3 && sizeof(T) == 4; }
     static size_t cand_smem(mg_tree *t, int l, Fields<T> &F, int cand) {
         const int n = t->lev[l].n, C = cells_of<D>(n), GH = 2 * D * face_of<D>(n);
         // stage of the kernels that read eps (k_sweep_warp, k_sweep_rows) and
@@ -4342,7 +4526,7 @@ template <class T, int D> struct Launch {
         const size_t stage_tma = F.W ? sizeof(BlockDesc) + sizeof(LevelDesc) + sizeof(T) * (2 * C + GH + (2 * D + 1) * C)
                                      : stage;
         switch (cand) {
-        case 0: return (n == 8 || n == 16) ? 2 * stage_tma : 0;
+        case 0: return n == 16 && rows16() ? kRows16Stages * stage : (n == 8 || n == 16) ? 2 * stage_tma : 0;
         case 10:  // half-width TMA sweep: only where it differs from candidate 0
             return ((n == 8 || n == 16) &&
                     sweep_tma_threads(cells_of<D>(n) / 2, true) != sweep_tma_threads(cells_of<D>(n) / 2, false))
@@ -4388,8 +4572,16 @@ template <class T, int D> struct Launch {
         switch (cand) {
         case 0: case 10: {
             const bool half = cand == 10;
+            if constexpr (rows16()) {
+                if (n == 16 && !half) {
+                    auto kern = F.E ? k_sweep_rows16<true> : k_sweep_rows16<false>;
+                    const int grid = std::min(nb, resident_ctas(kern, 512, sm) * t->nsm);
+                    launch_k(kern, grid, 512, sm, t->stream, P, L.first, nb, F, colour);
+                    return;
+                }
+            }
             auto kern = n == 8 ? (half ? k_sweep_tma<T, D, 8, true> : k_sweep_tma<T, D, 8>)
-                               : (half ? k_sweep_tma<T, D, 16, true> : k_sweep_tma<T, D, 16>);
+                               : (half || rows16() ? k_sweep_tma<T, D, 16, true> : k_sweep_tma<T, D, 16, rows16()>);
             const int thr = sweep_tma_threads(cells_of<D>(n) / 2, half);
             const int grid = std::min(nb, resident_ctas(kern, thr, sm) * t->nsm);
             launch_k(kern, grid, thr, sm, t->stream, P, L.first, nb, F, colour);
