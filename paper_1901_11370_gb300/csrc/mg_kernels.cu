@@ -2593,6 +2593,323 @@ __global__ void __launch_bounds__(128) k_restrict_rows(KParams P, int first, int
     }
 }
 
+// Quarter-row forms of the FP32 transfers of 3D 16^3 blocks with 16^3
+// parents, one 512-thread CTA per SM with three stages, as the sweep
+// (k_sweep_rows16): a thread takes two quarter rows (4 cells), their
+// neighbour rows come in with 16-byte loads, and the passes over shared
+// memory with a barrier each of k_restrict_tma and k_prolong_tma (child
+// residuals, octant values, the correction box) are gone.
+// Unit u of a block: q = u & 3, rows j = 2 (u >> 4 & 7) + (u >> 2 & 1) and
+// k = 2 (u >> 7) + (u >> 3 & 1), so that the four rows under a parent row
+// are lanes l, l ^ 4, l ^ 8, l ^ 12, and 8 lanes read 128 contiguous bytes.
+struct Row16 {
+    int q4, j, k, c;  // first cell, rows, its index in the block
+};
+__device__ __forceinline__ Row16 row16(int u) {
+    const int q4 = 4 * (u & 3), j = 2 * ((u >> 4) & 7) + ((u >> 2) & 1), k = 2 * (u >> 7) + ((u >> 3) & 1);
+    return Row16{q4, j, k, q4 + 16 * (j + 16 * k)};
+}
+
+template <bool VAR>
+__global__ void __launch_bounds__(512, 1) k_restrict_rows16(KParams P, int first, int nblocks, Fields<float> F) {
+    pdl_entry();
+    using T = float;
+    constexpr int n = 16, C = 4096, FC = 256, GH = 1536, ST = kRows16Stages;
+    constexpr int DESC = (int)((sizeof(BlockDesc) + sizeof(LevelDesc)) / sizeof(T));
+    constexpr int STAGE = 2 * DESC + 2 * C + GH + (VAR ? C + GH : 0);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bars[ST];
+    __shared__ int s_abort;
+    __shared__ __align__(16) T oct[512];  // parent cells under the block, [ck][cj][ci]
+    T *stage0 = reinterpret_cast<T *>(smem_raw);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        for (int q = 0; q < ST; q++) mbar_init(&bars[q], 1);
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    __syncthreads();
+    auto issue = [&](int it, int g) {  // thread 0 only; the offsets were read while earlier blocks were under way
+        T *st = stage0 + (it % ST) * STAGE;
+        uint64_t *bar = &bars[it % ST];
+        const BlockDesc &q = P.B[first + g];
+        const long long co = q.cell_off, go = q.ghost_off;
+        const int par = q.parent;
+        fence_async_smem();
+        mbar_expect_tx(bar, (uint32_t)(sizeof(T) * STAGE));
+        bulk_g2s(st, P.B + first + g, sizeof(BlockDesc), bar);
+        bulk_g2s(reinterpret_cast<char *>(st) + sizeof(BlockDesc), P.L + q.lev, sizeof(LevelDesc), bar);
+        bulk_g2s(st + DESC, P.B + par, sizeof(BlockDesc), bar);
+        bulk_g2s(reinterpret_cast<char *>(st + DESC) + sizeof(BlockDesc), P.L + P.B[par].lev, sizeof(LevelDesc), bar);
+        bulk_g2s(st + 2 * DESC, F.X + co, sizeof(T) * C, bar);
+        bulk_g2s(st + 2 * DESC + C, F.XG + go, sizeof(T) * GH, bar);
+        bulk_g2s_f<T>(st + 2 * DESC + C + GH, F.F + co, sizeof(T) * C, bar);
+        if (VAR) {
+            bulk_g2s_f<T>(st + 2 * DESC + 2 * C + GH, F.E + co, sizeof(T) * C, bar);
+            bulk_g2s_f<T>(st + 2 * DESC + 3 * C + GH, F.EG + go, sizeof(T) * GH, bar);
+        }
+    };
+    const int stride = gridDim.x;
+    int g = blockIdx.x;
+    if (tid == 0)
+        for (int q = 0; q < ST - 1; q++)
+            if (g + q * stride < nblocks) issue(q, g + q * stride);
+    const T helm = kp_helm<T>(P);
+    for (int it = 0; g < nblocks; it++, g += stride) {
+        if (!mbar_wait_bounded(&bars[it % ST], (it / ST) & 1, P.wait_limit)) {
+            atomicExch(P.status, 1);
+            s_abort = 1;
+        }
+        __syncthreads();
+        if (s_abort) {
+            // copies of this and the next blocks may still be landing in
+            // shared memory: let them arrive (normal bound) before the CTA exits
+            if (tid == 0)
+                for (int q = 0; q < ST - 1; q++)
+                    if (g + q * stride < nblocks)
+                        mbar_wait_bounded(&bars[(it + q) % ST], ((it + q) / ST) & 1, kWaitLimit);
+            break;
+        }
+        if (tid == 0 && g + (ST - 1) * stride < nblocks) issue(it + ST - 1, g + (ST - 1) * stride);
+        const T *st = stage0 + (it % ST) * STAGE;
+        const BlockDesc &b = *reinterpret_cast<const BlockDesc *>(st);
+        const BlockDesc &p = *reinterpret_cast<const BlockDesc *>(st + DESC);
+        const LevelDesc &L = *reinterpret_cast<const LevelDesc *>(reinterpret_cast<const char *>(st) + sizeof(BlockDesc));
+        const LevelDesc &PL = *reinterpret_cast<const LevelDesc *>(reinterpret_cast<const char *>(st + DESC) + sizeof(BlockDesc));
+        const T w0 = L.inv_h2f[0], w1 = L.inv_h2f[1], w2 = L.inv_h2f[2];
+        const T *xs = st + 2 * DESC, *fs = xs + C + GH, *es = fs + C;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const Row16 r = row16(tid + 512 * u);
+            const int dn = r.j > 0 ? r.c - n : C + 2 * FC + r.q4 + n * r.k, up = r.j < n - 1 ? r.c + n : C + 3 * FC + r.q4 + n * r.k;
+            const int bk = r.k > 0 ? r.c - n * n : C + 4 * FC + r.q4 + n * r.j;
+            const int fw = r.k < n - 1 ? r.c + n * n : C + 5 * FC + r.q4 + n * r.j;
+            const int lo = r.q4 > 0 ? r.c - 1 : C + r.j + n * r.k, hi = r.q4 < 12 ? r.c + 4 : C + FC + r.j + n * r.k;
+            auto row = [](const T *a, T *v) {
+                const float4 q = *reinterpret_cast<const float4 *>(a);
+                v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+            };
+            // (the ghosts follow the cells: one offset serves x and eps)
+            T x[6], xd[4], xu[4], xb[4], xf[4], f[4], res[4];
+            row(xs + r.c, x + 1);
+            x[0] = xs[lo];
+            x[5] = xs[hi];
+            row(xs + dn, xd);
+            row(xs + up, xu);
+            row(xs + bk, xb);
+            row(xs + fw, xf);
+            row(fs + r.c, f);
+            if (VAR) {
+                T e[6], ed[4], eu[4], eb[4], ef[4];
+                row(es + r.c, e + 1);
+                e[0] = es[lo];
+                e[5] = es[hi];
+                row(es + dn, ed);
+                row(es + up, eu);
+                row(es + bk, eb);
+                row(es + fw, ef);
+                T hx[5];  // (e e') / (e + e') of the faces along the row
+#pragma unroll
+                for (int q = 0; q < 5; q++) hx[q] = e[q] * __fdividef(e[q + 1], e[q] + e[q + 1]);
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const T xc = x[1 + q], ec = e[1 + q];
+                    T lx = hx[q] * (x[q] - xc);
+                    lx += hx[q + 1] * (x[q + 2] - xc);
+                    T ly = __fdividef(ed[q], ec + ed[q]) * (xd[q] - xc);
+                    ly += __fdividef(eu[q], ec + eu[q]) * (xu[q] - xc);
+                    T lz = __fdividef(eb[q], ec + eb[q]) * (xb[q] - xc);
+                    lz += __fdividef(ef[q], ec + ef[q]) * (xf[q] - xc);
+                    const T lap = (T)2 * (w0 * lx + ec * (w1 * ly + w2 * lz));
+                    res[q] = f[q] - (lap - helm * xc);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const T xc = x[1 + q];
+                    T lap = 0;
+                    lap += w0 * (x[q] - xc);
+                    lap += w0 * (x[q + 2] - xc);
+                    lap += w1 * (xd[q] - xc);
+                    lap += w1 * (xu[q] - xc);
+                    lap += w2 * (xb[q] - xc);
+                    lap += w2 * (xf[q] - xc);
+                    res[q] = f[q] - (lap - helm * xc);
+                }
+            }
+            T s4[4] = {x[1] + x[2], x[3] + x[4], res[0] + res[1], res[2] + res[3]};
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                s4[q] += __shfl_xor_sync(0xffffffffu, s4[q], 4);
+                s4[q] += __shfl_xor_sync(0xffffffffu, s4[q], 8);
+            }
+            if (!(r.j & 1) && !(r.k & 1)) {
+                const int ci = r.q4 / 2, cj = r.j >> 1, ck = r.k >> 1;
+                const T inv = (T)(1.0 / 8);
+                const int pc = cidx<3>(n, b.poff[0] + ci, b.poff[1] + cj, b.poff[2] + ck);
+                const float2 xv = make_float2(s4[0] * inv, s4[1] * inv);
+                *reinterpret_cast<float2 *>(F.X + p.cell_off + pc) = xv;
+                *reinterpret_cast<float2 *>(F.F + p.cell_off + pc) = make_float2(s4[2] * inv, s4[3] * inv);
+                *reinterpret_cast<float2 *>(oct + (ck * 8 + cj) * 8 + ci) = xv;
+            }
+        }
+        __syncthreads();
+        // parent ghosts beside the octant: faces where it meets the parent's boundary
+        for (int t = tid; t < 6 * 64; t += 512) {
+            const int face = t >> 6, v = t & 63, d = face >> 1, s = face & 1;
+            const int off = d == 0 ? b.poff[0] : d == 1 ? b.poff[1] : b.poff[2];
+            if (!(s ? (off + 8 == n) : (off == 0))) continue;
+            const int a = v & 7, c = v >> 3, e = s ? 7 : 0, e2 = s ? 6 : 1;  // octant-local
+            const I3 lo = d == 0 ? I3{e, a, c} : (d == 1 ? I3{a, e, c} : I3{a, c, e});
+            const I3 li = d == 0 ? I3{e2, a, c} : (d == 1 ? I3{a, e2, c} : I3{a, c, e2});
+            const I3 ii{b.poff[0] + lo.x, b.poff[1] + lo.y, b.poff[2] + lo.z};
+            const int w = d == 0 ? ii.y + n * ii.z : (d == 1 ? ii.x + n * ii.z : ii.x + n * ii.y);
+            const T cv = oct[(lo.z * 8 + lo.y) * 8 + lo.x];
+            const int nb = p.nbr[face];
+            if (nb >= 0) F.XG[p.push[face] + w] = cv;
+            else if (nb == -1) F.XG[p.ghost_off + face * FC + w] = phys_ghost<T>(P, PL, face, cv, bc_value(P, PL, p, 3, face, ii));
+            else
+                F.XG[p.ghost_off + face * FC + w] =
+                    cf_ghost<T, 3>(P, PL, p, face, ii, cv, oct[(li.z * 8 + li.y) * 8 + li.x], F.X, F.XG, nb, false);
+        }
+        // the next iteration's wait barrier orders these reads of oct and the
+        // stage before their next use
+    }
+}
+
+__global__ void __launch_bounds__(512, 1) k_prolong_rows16(KParams P, int first, int nblocks, Fields<float> F) {
+    pdl_entry();
+    using T = float;
+    constexpr int n = 16, C = 4096, FC = 256, GH = 1536, ST = kRows16Stages;
+    constexpr int DESC = (int)((sizeof(BlockDesc) + sizeof(LevelDesc)) / sizeof(T));
+    constexpr int PD = (int)(sizeof(BlockDesc) / sizeof(T));
+    constexpr int STAGE = DESC + PD + C + 2 * (C + GH);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bars[ST];
+    __shared__ int s_abort;
+    T *stage0 = reinterpret_cast<T *>(smem_raw);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        for (int q = 0; q < ST; q++) mbar_init(&bars[q], 1);
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    __syncthreads();
+    auto issue = [&](int it, int g) {  // thread 0 only
+        T *st = stage0 + (it % ST) * STAGE;
+        uint64_t *bar = &bars[it % ST];
+        const BlockDesc &q = P.B[first + g];
+        const long long co = q.cell_off;
+        const int par = q.parent;
+        const long long pco = P.B[par].cell_off, pgo = P.B[par].ghost_off;
+        fence_async_smem();
+        mbar_expect_tx(bar, (uint32_t)(sizeof(T) * STAGE));
+        bulk_g2s(st, P.B + first + g, sizeof(BlockDesc), bar);
+        bulk_g2s(reinterpret_cast<char *>(st) + sizeof(BlockDesc), P.L + q.lev, sizeof(LevelDesc), bar);
+        bulk_g2s(st + DESC, P.B + par, sizeof(BlockDesc), bar);
+        T *d = st + DESC + PD;
+        bulk_g2s(d, F.X + co, sizeof(T) * C, bar);
+        bulk_g2s(d + C, F.X + pco, sizeof(T) * C, bar);
+        bulk_g2s(d + 2 * C, F.XG + pgo, sizeof(T) * GH, bar);
+        bulk_g2s(d + 2 * C + GH, F.V + pco, sizeof(T) * C, bar);
+        bulk_g2s(d + 3 * C + GH, F.VG + pgo, sizeof(T) * GH, bar);
+    };
+    const int stride = gridDim.x;
+    int g = blockIdx.x;
+    if (tid == 0)
+        for (int q = 0; q < ST - 1; q++)
+            if (g + q * stride < nblocks) issue(q, g + q * stride);
+    for (int it = 0; g < nblocks; it++, g += stride) {
+        if (!mbar_wait_bounded(&bars[it % ST], (it / ST) & 1, P.wait_limit)) {
+            atomicExch(P.status, 1);
+            s_abort = 1;
+        }
+        __syncthreads();
+        if (s_abort) {
+            // copies of this and the next blocks may still be landing in
+            // shared memory: let them arrive (normal bound) before the CTA exits
+            if (tid == 0)
+                for (int q = 0; q < ST - 1; q++)
+                    if (g + q * stride < nblocks)
+                        mbar_wait_bounded(&bars[(it + q) % ST], ((it + q) / ST) & 1, kWaitLimit);
+            break;
+        }
+        if (tid == 0 && g + (ST - 1) * stride < nblocks) issue(it + ST - 1, g + (ST - 1) * stride);
+        T *st = stage0 + (it % ST) * STAGE;
+        const BlockDesc &b = *reinterpret_cast<const BlockDesc *>(st);
+        const LevelDesc &L = *reinterpret_cast<const LevelDesc *>(reinterpret_cast<const char *>(st) + sizeof(BlockDesc));
+        T *xs = st + DESC + PD;
+        // parent x then its ghosts, x_old then its ghosts: one offset serves both pairs
+        const T *px = xs + C, *pv = px + C + GH;
+        const int cfm = cf_faces(b, 3);
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const Row16 r = row16(tid + 512 * u);
+            // parent cells p0, p0 + 1 of row (pj, pk), their x neighbours, and
+            // the two cells of the rows on the cells' y and z sides
+            const int p0 = b.poff[0] + r.q4 / 2, pj = b.poff[1] + (r.j >> 1), pk = b.poff[2] + (r.k >> 1);
+            const int qj = pj + ((r.j & 1) ? 1 : -1), qk = pk + ((r.k & 1) ? 1 : -1);
+            const int row = n * (pj + n * pk);
+            const int im = p0 > 0 ? row + p0 - 1 : C + pj + n * pk, ip = p0 + 2 < n ? row + p0 + 2 : C + FC + pj + n * pk;
+            const int iy = qj < 0 ? C + 2 * FC + n * pk + p0 : qj >= n ? C + 3 * FC + n * pk + p0 : n * (qj + n * pk) + p0;
+            const int iz = qk < 0 ? C + 4 * FC + n * pj + p0 : qk >= n ? C + 5 * FC + n * pj + p0 : n * (pj + n * qk) + p0;
+            auto d1 = [&](int i) { return px[i] - pv[i]; };
+            auto d2 = [&](int i) {  // p0 is even
+                const float2 a = *reinterpret_cast<const float2 *>(px + i), o = *reinterpret_cast<const float2 *>(pv + i);
+                return make_float2(a.x - o.x, a.y - o.y);
+            };
+            const float2 x01 = d2(row + p0), y01 = d2(iy), z01 = d2(iz);
+            const T xm = d1(im), xp = d1(ip);
+            float4 v = *reinterpret_cast<const float4 *>(xs + r.c);
+            v.x += (x01.x + (xm + y01.x + z01.x)) * 0.25f;
+            v.y += (x01.x + (x01.y + y01.x + z01.x)) * 0.25f;
+            v.z += (x01.y + (x01.x + y01.y + z01.y)) * 0.25f;
+            v.w += (x01.y + (xp + y01.y + z01.y)) * 0.25f;
+            *reinterpret_cast<float4 *>(F.X + b.cell_off + r.c) = v;
+            if (cfm) *reinterpret_cast<float4 *>(xs + r.c) = v;
+            // same-level and physical ghosts of these cells, from registers
+            if (r.q4 == 0 || r.q4 == 12) {
+                const int fx = r.q4 ? 1 : 0, nb = b.nbr[fx];
+                const T ve = r.q4 ? v.w : v.x;
+                if (nb >= 0) F.XG[b.push[fx] + r.j + n * r.k] = ve;
+                else if (nb == -1)
+                    F.XG[b.ghost_off + fx * FC + r.j + n * r.k] =
+                        phys_ghost<T>(P, L, fx, ve, bc_value(P, L, b, 3, fx, I3{r.q4 ? n - 1 : 0, r.j, r.k}));
+            }
+            auto face4 = [&](int face, int t1) {  // 4 cells, contiguous on the face; t1: their second coordinate
+                const int nb = b.nbr[face], u0 = r.q4 + n * t1;
+                if (nb >= 0) {
+                    *reinterpret_cast<float4 *>(F.XG + b.push[face] + u0) = v;
+                } else if (nb == -1) {
+                    const int d = face >> 1, edge = (face & 1) ? n - 1 : 0;
+                    const T w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const I3 ii = d == 1 ? I3{r.q4 + q, edge, t1} : I3{r.q4 + q, t1, edge};
+                        F.XG[b.ghost_off + face * FC + u0 + q] = phys_ghost<T>(P, L, face, w[q], bc_value(P, L, b, 3, face, ii));
+                    }
+                }
+            };
+            if (r.j == 0 || r.j == n - 1) face4(r.j ? 3 : 2, r.k);
+            if (r.k == 0 || r.k == n - 1) face4(r.k ? 5 : 4, r.j);
+        }
+        if (cfm) {
+            __syncthreads();  // the updated rows in the stage
+            for (int t = tid; t < GH; t += 512) {
+                const int face = t / FC, u = t - face * FC;
+                if (!((cfm >> face) & 1)) continue;
+                const I3 ii = face_cell<3>(n, face, u, false);
+                I3 dd = ii;
+                put(dd, face >> 1, (face & 1) ? n - 2 : 1);
+                F.XG[b.ghost_off + t] = cf_ghost<T, 3>(P, L, b, face, ii, xs[cidx<3>(n, ii.x, ii.y, ii.z)],
+                                                       xs[cidx<3>(n, dd.x, dd.y, dd.z)], F.X, F.XG, b.nbr[face], false);
+            }
+        }
+        // the next iteration's wait barrier orders this block's stage reads
+        // before the stage's refill
+    }
+}
+
 // ---------------------------------------------- divergence cleaning -----
 // Second-order central differences on leaf blocks (Sec. 4.1): component d of
 // a vector field X (with ghosts) adds (X(c+e_d) - X(c-e_d)) / (2 h_d) to the
@@ -4751,6 +5068,16 @@ template <class T, int D> struct Launch {
         const int C8 = cells_of<D>(L.n), GH8 = 2 * D * face_of<D>(L.n);
         const size_t smt = 2 * (2 * (sizeof(BlockDesc) + sizeof(LevelDesc)) +
                                 sizeof(T) * (2 * C8 + GH8 + (F.W ? 2 * D * C8 : (F.E ? C8 + GH8 : 0))));
+        if constexpr (rows16()) {
+            const size_t s16 = kRows16Stages * (2 * (sizeof(BlockDesc) + sizeof(LevelDesc)) +
+                                                sizeof(T) * (2 * C8 + GH8 + (F.E ? C8 + GH8 : 0)));
+            if (L.n == 16 && L.parent_same_n) {
+                auto kern = F.E ? k_restrict_rows16<true> : k_restrict_rows16<false>;
+                const int grid = std::min(L.nb, resident_ctas(kern, 512, s16) * t->nsm);
+                launch_k(kern, grid, 512, s16, t->stream, P, L.first, L.nb, F);
+                return;
+            }
+        }
         if (D == 3 && L.n == 8 && L.parent_same_n && !F.W && !F.E && t->geom == MG_CART) {
             const size_t sr = 2 * sizeof(T) * (2 * C8 + GH8) + 4 * (sizeof(BlockDesc) + sizeof(LevelDesc));
             set_smem(k_restrict_rows<T>, sr);
@@ -4849,6 +5176,14 @@ template <class T, int D> struct Launch {
     static void prolong(mg_tree *t, const KParams &P, int l, Fields<T> &F) {
         const LevelHost &L = t->lev[l];
         ++t->launches;
+        if constexpr (rows16()) {
+            if (L.n == 16 && L.parent_same_n) {
+                const size_t s16 = kRows16Stages * (prolong_tma_smem(L) / 2);
+                const int grid = std::min(L.nb, resident_ctas(k_prolong_rows16, 512, s16) * t->nsm);
+                launch_k(k_prolong_rows16, grid, 512, s16, t->stream, P, L.first, L.nb, F);
+                return;
+            }
+        }
         if (D == 3 && L.n == 8 && L.parent_same_n) {
             const size_t smt = prolong_tma_smem(L);
             set_smem(k_prolong_rows<T>, smt);
