@@ -75,7 +75,8 @@ enum { MG_SMOOTH_RBGS = 0, MG_SMOOTH_JACOBI = 1 };
  * V-cycles per outer FP64 residual.  smoother MG_SMOOTH_RBGS or
  * MG_SMOOTH_JACOBI; omega the Jacobi weight (<= 0: 4/5 in 2D, 6/7 in 3D;
  * at most 1).  coarse_mode MG_COARSE_EXACT solves the coarsest level
- * exactly (a dense FP64 inverse; in a batch, the block-tridiagonal form
+ * exactly (a dense FP64 inverse, or the operator's eigenvectors with a
+ * constant coefficient; in a batch, the block-tridiagonal form
  * described at mg_batch_create, FP32 inside FP32 cycles); MG_COARSE_SMOOTH
  * is the paper's coarse-grid
  * solve: red-black Gauss-Seidel sweeps of the coarsest level (FP64) until
@@ -236,6 +237,9 @@ int mg_residual_norm(mg_tree *t, double *l2, double *linf, double *dev_r);
  * and adds e to phi in FP64.  *cycles_done counts outer steps, *rel_out the
  * final relative residual.  On a singular problem phi is returned with zero
  * volume-weighted mean.  Returns MG_ERR_NOT_CONVERGED at max_cycles.
+ * On a single Cartesian tree the levels below the base grid (and small base
+ * grids) run in one thread-block-cluster launch per cycle leg, the same
+ * cycle up to rounding order; mg_vcycle and mg_fmg run launch by launch.
  */
 int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_first,
              const mg_params *p, int *cycles_done, double *rel_out);
@@ -399,7 +403,8 @@ int mg_set_wait_limit(mg_tree *t, int64_t polls);
  * (level -1: on every level where it applies; variant -1: back to the
  * automatic choice).  MG_ERR_ARG when a single level is named and the
  * variant does not apply there.  Every variant computes the same red-black
- * half-sweep; this call exists to test and time them one by one. */
+ * half-sweep; this call exists to test and time them one by one.  While a
+ * variant is pinned, solves run launch by launch on every level. */
 int mg_sweep_variant(mg_tree *t, int precision, int level, int *variant);
 int mg_set_sweep_variant(mg_tree *t, int precision, int level, int variant);
 /* mg_set_tail: an option for the small levels at the bottom of a V-cycle
