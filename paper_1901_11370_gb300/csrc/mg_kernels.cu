@@ -2995,9 +2995,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_grad_sub(KParams P, int first, 
 // block size at compile time and kMaxThreads threads, so that a thread's
 // cells form a fixed loop the compiler unrolls (the loads of several cells
 // are in flight before their FP64 arithmetic, which on GB300 holds a warp
-// for many cycles per instruction).
+// for many cycles per instruction).  Its floor at 16.8M cells with variable
+// eps is 370 us of FP64 issue (13 instructions a cell) and 190 us of bytes;
+// it is between the two and load latency, so the split is a matter of warps
+// against loads in flight.  The 256^3 solve (17 launches): three CTAs a SM
+// 54.2 ms, four 52.6; four without unrolling 54.6; two with four cells
+// unrolled 58.4.
 template <int D, bool MX = true, int NT = 0>
-__global__ void __launch_bounds__(kMaxThreads, NT ? 3 : 2) k_resnorm(KParams P, int first, Fields<double> F,
+__global__ void __launch_bounds__(kMaxThreads, NT ? 4 : 2) k_resnorm(KParams P, int first, Fields<double> F,
                                                          double *__restrict__ partials,
                                                          double *__restrict__ rleaf, long long leaf_base,
                                                          long long cell_base, float *__restrict__ f32) {
