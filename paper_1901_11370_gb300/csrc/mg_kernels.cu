@@ -2292,7 +2292,7 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
             // of a parent cell share their inner faces, whose fluxes cancel.
             // What is left is sum_d w_d (outer neighbours in d - children):
             // 5 instead of 16 FP64 instructions a child in 3D, and no pass
-            // over the child residuals (128^3 Jacobi solve: 44 -> 20 us a launch).
+            // over the child residuals (128^3 Jacobi solve: 44 -> 23 us a launch).
             if (!var && !cyl) {
                 done = true;
                 const T wsum = ih0 + ih1 + (D == 3 ? ih2 : (T)0) + kp_helm<T>(P), inv = (T)(1.0 / (1 << D));
