@@ -919,6 +919,7 @@ template <class T, int D>
 __global__ void __launch_bounds__(256) k_bottom_coef(BotPlan B, int l, const int *__restrict__ bmap, int n, int nbx,
                                                      int nby, long long cell_first, const double *__restrict__ W,
                                                      T *__restrict__ out) {
+    pdl_entry();
     const int A = B.n0[0] << l, NB = D == 3 ? B.n0[1] << l : 1, NP = B.n0[2] << l, C = cells_of<D>(n);
     const long long cells = (long long)A * NB * NP;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < cells; c += (long long)gridDim.x * blockDim.x) {

@@ -35,6 +35,7 @@ template <int D>
 __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, const int *__restrict__ map,
                                                      const double *__restrict__ E, double sigma, int ld,
                                                      double *__restrict__ A, int *__restrict__ flag) {
+    pdl_entry();
     const int row = blockIdx.x * blockDim.x + threadIdx.x, C = cells_of<D>(tc.n);
     if (row >= tc.nc) return;
     const BlockDesc &b = P.B[tc.first + row / C];
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, c
 __global__ void __launch_bounds__(kPanelThreads) k_inv_panel(const double *__restrict__ A, int n, int ld, int at,
                                                              double *__restrict__ R, double *__restrict__ Cc,
                                                              int *__restrict__ flag) {
+    pdl_entry();
     __shared__ double S[kPanel][kPanel + 1], T[kPanel][kTile + 1];
     const int nb = min(kPanel, n - at), tid = threadIdx.x, c0 = blockIdx.x * kTile;
     for (int e = tid; e < kPanel * kPanel; e += kPanelThreads) {
@@ -150,6 +152,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_inv_panel(const double *__res
 __global__ void __launch_bounds__(kPanelThreads) k_inv_update(double *__restrict__ A, int n, int ld, int at,
                                                               const double *__restrict__ R,
                                                               const double *__restrict__ Cc) {
+    pdl_entry();
     __shared__ double X[kTile][kPanel + 1], Y[kPanel][kTile + 1];
     const int nb = min(kPanel, n - at), tid = threadIdx.x, r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
     for (int e = tid; e < kTile * kPanel; e += kPanelThreads) {
@@ -186,6 +189,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_inv_update(double *__restrict
 template <int D>
 __global__ void __launch_bounds__(256) k_inv_store(KParams P, TreeCoarse tc, const double *__restrict__ A, int ld,
                                                    double sigma, double vsum, double *__restrict__ minv) {
+    pdl_entry();
     const long long total = (long long)tc.nc * tc.ns;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         const int row = (int)(e / tc.ns), c = (int)(e % tc.ns);

@@ -5754,6 +5754,7 @@ __global__ void __launch_bounds__(256) k_transfer(const BlockDesc *__restrict__ 
                                                   const double *__restrict__ OXG, const BlockDesc *__restrict__ NB,
                                                   const int *__restrict__ nid, const int *__restrict__ src,
                                                   double *__restrict__ NX) {
+    pdl_entry();
     const BlockDesc &b = NB[nid[blockIdx.x]];
     const int s = src[blockIdx.x], n = b.n, C = cells_of<D>(n);
     if (s >= 0) {
