@@ -290,8 +290,8 @@ template <class T, int D, bool VAR> struct Bottom {
         cluster_sync();
     }
     __device__ __forceinline__ T ih(int l, int i) const { return lv_ih<T>(L[l], B.perm[i]); }
-    // L x - lambda x at a cell of level q (difference form in FP32, whose
-    // rounding follows the differences; sum form in FP64)
+    // L x - lambda x at a cell of level q, in differences: their rounding
+    // follows w |dx|, that of a sum form w |x|
     __device__ __forceinline__ T lap(const BotLev<T, D> &q, int a, int b, int p, T w0, T w1, T w2) const {
         const T *x = q.X + q.at(a, b, p);
         const T xc = x[0];
@@ -307,22 +307,15 @@ template <class T, int D, bool VAR> struct Bottom {
             s += w[(2 * D - 1) * q.wn] * (x[q.SP] - xc);
             return s - kp_helm<T>(P) * xc;
         }
-        if constexpr (sizeof(T) == 8) {
-            T s = w0 * (x[-1] + x[1]);
-            if (D == 3) s += w1 * (x[-q.SA] + x[q.SA]);
-            s += w2 * (x[-q.SP] + x[q.SP]);
-            return s - (T)L[q.l].diag * xc;
-        } else {
-            T s = w0 * (x[-1] - xc);
-            s += w0 * (x[1] - xc);
-            if (D == 3) {
-                s += w1 * (x[-q.SA] - xc);
-                s += w1 * (x[q.SA] - xc);
-            }
-            s += w2 * (x[-q.SP] - xc);
-            s += w2 * (x[q.SP] - xc);
-            return s - kp_helm<T>(P) * xc;
+        T s = w0 * (x[-1] - xc);
+        s += w0 * (x[1] - xc);
+        if (D == 3) {
+            s += w1 * (x[-q.SA] - xc);
+            s += w1 * (x[q.SA] - xc);
         }
+        s += w2 * (x[-q.SP] - xc);
+        s += w2 * (x[q.SP] - xc);
+        return s - kp_helm<T>(P) * xc;
     }
     // the local Gauss-Seidel solution at padded index i (Sec. 2.2); wi: its coefficient index
     __device__ __forceinline__ T local_at(const BotLev<T, D> &q, int i, int wi, T w0, T w1, T w2, T idiag) const {
@@ -458,8 +451,9 @@ template <class T, int D, bool VAR> struct Bottom {
             T sx = 0, sr = 0;
             if (sizeof(T) == 8 && !VAR) {
                 // FP64: the Laplacians of the 2^D children share their inner
-                // faces, whose fluxes cancel: sum_d w_d (outer neighbours in d
-                // - children).  5 instead of 13 FP64 instructions a child.
+                // faces, whose fluxes cancel: sum_d w_d sum (outer neighbour
+                // in d - child), the differences kept (see k_restrict_tma).
+                // 8 instead of 16 FP64 instructions a child.
                 T oa = 0, ob = 0, op = 0;
                 const T *x = q.X + q.at(fa, fb, fp);
                 const T *f = q.F + q.fat(fa, fb, fp);
@@ -468,19 +462,22 @@ template <class T, int D, bool VAR> struct Bottom {
 #pragma unroll
                     for (int g = 0; g < 2; g++) {  // the row of children at b + e, p + g
                         const T *y = x + e * q.SA + g * q.SP;
-                        const T pair = y[0] + y[1];
-                        sx += pair;
-                        oa += y[-1] + y[2];
-                        if (D == 3) ob += e ? y[q.SA] + y[q.SA + 1] : y[-q.SA] + y[-q.SA + 1];
-                        op += g ? y[q.SP] + y[q.SP + 1] : y[-q.SP] + y[-q.SP + 1];
+                        const T y0 = y[0], y1 = y[1];
+                        sx += y0 + y1;
+                        oa += (y[-1] - y0) + (y[2] - y1);
+                        if (D == 3) {
+                            const T *o = y + (e ? q.SA : -q.SA);
+                            ob += (o[0] - y0) + (o[1] - y1);
+                        }
+                        const T *o = y + (g ? q.SP : -q.SP);
+                        op += (o[0] - y0) + (o[1] - y1);
                         const T *fr = f + e * q.SA + g * q.SP;
                         sr += fr[0] + fr[1];
                     }
-                const T wsum = w0 + (D == 3 ? w1 : (T)0) + w2 + helm;
-                T s = fma(-w0, oa, sr);
+                T s = fma(helm, sx, sr);
+                s = fma(-w0, oa, s);
                 if (D == 3) s = fma(-w1, ob, s);
-                s = fma(-w2, op, s);
-                sr = fma(wsum, sx, s);
+                sr = fma(-w2, op, s);
             } else {
 #pragma unroll
                 for (int ch = 0; ch < (1 << D); ch++) {

@@ -2290,12 +2290,16 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
         if constexpr (sizeof(T) == 8) {
             // FP64, constant coefficient: the Laplacians of the 2^D children
             // of a parent cell share their inner faces, whose fluxes cancel.
-            // What is left is sum_d w_d (outer neighbours in d - children):
-            // 5 instead of 16 FP64 instructions a child in 3D, and no pass
-            // over the child residuals (128^3 Jacobi solve: 44 -> 23 us a launch).
+            // What is left is sum_d w_d sum (outer neighbour in d - child).
+            // The differences are kept: sums of neighbours minus sums of
+            // children would take a third less FP64, but their rounding
+            // follows w |x| instead of w |dx|, alike in cells of like x, and
+            // the coarse grids amplify it by 1 / (h^2 lambda_min) (2D 1024^2,
+            // x = 1e4: error 1399 instead of 10 units of rounding; 128^3
+            // Jacobi solve 8.89 against 9.27 ms).
             if (!var && !cyl) {
                 done = true;
-                const T wsum = ih0 + ih1 + (D == 3 ? ih2 : (T)0) + kp_helm<T>(P), inv = (T)(1.0 / (1 << D));
+                const T inv = (T)(1.0 / (1 << D));
                 for (int c = tid; c < M; c += nth) {
                     const int ci = c % m, cj = (c / m) % m, ck = D == 3 ? c / (m * m) : 0;
                     T sx = 0, sf = 0, ox = 0, oy = 0, oz = 0;
@@ -2304,13 +2308,14 @@ __global__ void __launch_bounds__(transfer_bound(D, NT), (D == 3 && NT == 16) ? 
 #pragma unroll
                         for (int e = 0; e < 2; e++) {  // the row of two children at j + e, k + g
                             const int i = 2 * ci, j = 2 * cj + e, k = D == 3 ? 2 * ck + g : 0, fc = cidx<D>(n, i, j, k);
-                            sx += xs[fc] + xs[fc + 1];
+                            const T x0 = xs[fc], x1 = xs[fc + 1];
+                            sx += x0 + x1;
                             sf += fs[fc] + fs[fc + 1];
-                            ox += nbv(xs, gs, i, j, k, 0, 0) + nbv(xs, gs, i + 1, j, k, 0, 1);
-                            oy += nbv(xs, gs, i, j, k, 1, e) + nbv(xs, gs, i + 1, j, k, 1, e);
-                            if (D == 3) oz += nbv(xs, gs, i, j, k, 2, g) + nbv(xs, gs, i + 1, j, k, 2, g);
+                            ox += (nbv(xs, gs, i, j, k, 0, 0) - x0) + (nbv(xs, gs, i + 1, j, k, 0, 1) - x1);
+                            oy += (nbv(xs, gs, i, j, k, 1, e) - x0) + (nbv(xs, gs, i + 1, j, k, 1, e) - x1);
+                            if (D == 3) oz += (nbv(xs, gs, i, j, k, 2, g) - x0) + (nbv(xs, gs, i + 1, j, k, 2, g) - x1);
                         }
-                    T r = fma(wsum, sx, sf);
+                    T r = fma(kp_helm<T>(P), sx, sf);
                     r = fma(-ih0, ox, r);
                     r = fma(-ih1, oy, r);
                     if (D == 3) r = fma(-ih2, oz, r);
@@ -2517,18 +2522,18 @@ __global__ void __launch_bounds__(128) k_restrict_rows(KParams P, int first, int
         ld4(fs + 8 * r + 4 * h, f4);
         T s4[4];
         if constexpr (sizeof(T) == 8) {
-            // the inner faces of the 2x2x2 children cancel (see
-            // k_restrict_tma): of each row only the outer y and z neighbours
-            // and both ends of the cell pairs count.  26 instead of 68 FP64
-            // instructions a thread.
-            const T wsum = w0 + w1 + w2 + helm;
+            // the inner faces of the 2x2x2 children cancel, the differences
+            // over the outer ones are kept (see k_restrict_tma): of each row
+            // only the outer y and z neighbours and both ends of the cell
+            // pairs count.  38 instead of 68 FP64 instructions a thread.
 #pragma unroll
             for (int q = 0; q < 2; q++) {
-                s4[q] = xr[1 + 2 * q] + xr[2 + 2 * q];
-                T rr = fma(wsum, s4[q], f4[2 * q] + f4[2 * q + 1]);
-                rr = fma(-w0, xr[2 * q] + xr[3 + 2 * q], rr);
-                rr = fma(-w1, oy[2 * q] + oy[2 * q + 1], rr);
-                s4[2 + q] = fma(-w2, oz[2 * q] + oz[2 * q + 1], rr);
+                const T x0 = xr[1 + 2 * q], x1 = xr[2 + 2 * q];
+                s4[q] = x0 + x1;
+                T rr = fma(helm, s4[q], f4[2 * q] + f4[2 * q + 1]);
+                rr = fma(-w0, (xr[2 * q] - x0) + (xr[3 + 2 * q] - x1), rr);
+                rr = fma(-w1, (oy[2 * q] - x0) + (oy[2 * q + 1] - x1), rr);
+                s4[2 + q] = fma(-w2, (oz[2 * q] - x0) + (oz[2 * q + 1] - x1), rr);
             }
         } else {
             T res[4];
