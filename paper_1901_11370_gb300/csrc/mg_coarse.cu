@@ -13,6 +13,10 @@
 // [A 1; V^T 0] that the host inverts, the solves use the rows of the cells:
 // with K = (A - sigma 1 V^T)^-1, v = sum V and A 1 = 0, V^T A = 0 they are
 //   K + 1 V^T / (sigma v^2)   and, in the border's column,   1 / v.
+// sigma = max |A_ii| / v: the constants move to the operator's own size.  A
+// shift of the size of 1 / h^2 alone left K's constant part, or A, with too
+// few digits where eps is far from 1 (residual of the solve with 1 .. 10
+// times 1e12: 1e-4 of the right-hand side, now 7e-15; bordered 3e-15).
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -27,14 +31,27 @@ constexpr int kPanel = 32;          // pivot block
 constexpr int kPanelThreads = 256;
 constexpr int kTile = 32;           // update tile, kPanelThreads threads, 2 x 2 values each
 
+// volume of coarsest cell c (block order)
+template <int D> __device__ __forceinline__ double coarse_vol(const KParams &P, const TreeCoarse &tc, int c) {
+    const BlockDesc &b = P.B[tc.first + c / cells_of<D>(tc.n)];
+    const LevelDesc &L = P.L[b.lev];
+    if (P.geom != MG_CYL) return L.vol;
+    return 2.0 * M_PI * (P.lo[0] + (b.ijk[0] * tc.n + c % tc.n + 0.5) * L.h[0]) * L.h[0] * L.h[1];
+}
+// sigma from the largest |A_ii| (a single cell that couples to nothing has 0: any shift will do)
+__device__ __forceinline__ double coarse_shift(const CoarseInfo *info, double vsum) {
+    const double m = __longlong_as_double((long long)info->amax);
+    return (m > 0.0 ? m : 1.0) / vsum;
+}
+
 // A's row of every coarsest cell, row by row (one thread each; the matrix was
 // zeroed): rows and columns in block order, `map` from the cell's global
 // index to its row.  flag 2: a coefficient that is not positive (the host
 // inverts such a matrix, with pivoting).
 template <int D>
 __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, const int *__restrict__ map,
-                                                     const double *__restrict__ E, double sigma, int ld,
-                                                     double *__restrict__ A, int *__restrict__ flag) {
+                                                     const double *__restrict__ E, int ld, double *__restrict__ A,
+                                                     CoarseInfo *__restrict__ info) {
     pdl_entry();
     const int row = blockIdx.x * blockDim.x + threadIdx.x, C = cells_of<D>(tc.n);
     if (row >= tc.nc) return;
@@ -44,7 +61,7 @@ __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, c
     cell_of(row % C, tc.n, D, i, j, k);
     const I3 g{b.ijk[0] * tc.n + i, b.ijk[1] * tc.n + j, D == 3 ? b.ijk[2] * tc.n + k : 0};
     const double ri = P.lo[0] + (g.x + 0.5) * L.h[0], ec = E ? E[tc.cell0 + row] : 1.0;
-    if (!(ec > 0.0)) *flag = 2;
+    if (!(ec > 0.0)) info->flag = 2;
     double *a = A + (long long)row * ld;
     double diag = -P.helm;
 #pragma unroll
@@ -75,14 +92,19 @@ __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, c
             }
         }
     a[row] += diag;
-    if (!tc.singular) return;
-    double vol = L.vol;
-    for (int c = 0; c < tc.nc; c++) {  // - sigma V_c
-        if (P.geom == MG_CYL) {
-            const BlockDesc &o = P.B[tc.first + c / C];
-            vol = 2.0 * M_PI * (P.lo[0] + (o.ijk[0] * tc.n + c % tc.n + 0.5) * L.h[0]) * L.h[0] * L.h[1];
-        }
-        a[c] -= sigma * vol;
+    if (tc.singular) atomicMax(&info->amax, (unsigned long long)__double_as_longlong(fabs(diag)));  // >= 0: ordered as integers
+}
+
+// The shift of a singular system: - sigma V_c in column c of every row.
+template <int D>
+__global__ void __launch_bounds__(256) k_coarse_shift(KParams P, TreeCoarse tc, int ld, double vsum,
+                                                      const CoarseInfo *__restrict__ info, double *__restrict__ A) {
+    pdl_entry();
+    const double sigma = coarse_shift(info, vsum);
+    const long long total = (long long)tc.nc * tc.nc;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const int row = (int)(e / tc.nc), c = (int)(e % tc.nc);
+        A[(long long)row * ld + c] -= sigma * coarse_vol<D>(P, tc, c);
     }
 }
 
@@ -93,7 +115,7 @@ __global__ void __launch_bounds__(128) k_coarse_rows(KParams P, TreeCoarse tc, c
 // columns); and copies its share of the pivot columns.
 __global__ void __launch_bounds__(kPanelThreads) k_inv_panel(const double *__restrict__ A, int n, int ld, int at,
                                                              double *__restrict__ R, double *__restrict__ Cc,
-                                                             int *__restrict__ flag) {
+                                                             CoarseInfo *__restrict__ info) {
     pdl_entry();
     __shared__ double S[kPanel][kPanel + 1], T[kPanel][kTile + 1];
     const int nb = min(kPanel, n - at), tid = threadIdx.x, c0 = blockIdx.x * kTile;
@@ -116,7 +138,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_inv_panel(const double *__res
     const int r = tid >> 3, cb = (tid & 7) * 4;
     for (int p = 0; p < nb; p++) {
         const double ip = s_ip[p & 1], g = -S[r][p] * ip;
-        if (tid == 0 && blockIdx.x == 0 && S[p][p] == 0.0) atomicMax(flag, 1);
+        if (tid == 0 && blockIdx.x == 0 && S[p][p] == 0.0) atomicMax(&info->flag, 1);
         double v[4];
 #pragma unroll
         for (int e = 0; e < 4; e++) {
@@ -188,7 +210,8 @@ __global__ void __launch_bounds__(kPanelThreads) k_inv_update(double *__restrict
 // border's column.
 template <int D>
 __global__ void __launch_bounds__(256) k_inv_store(KParams P, TreeCoarse tc, const double *__restrict__ A, int ld,
-                                                   double sigma, double vsum, double *__restrict__ minv) {
+                                                   double vsum, const CoarseInfo *__restrict__ info,
+                                                   double *__restrict__ minv) {
     pdl_entry();
     const long long total = (long long)tc.nc * tc.ns;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
@@ -198,14 +221,7 @@ __global__ void __launch_bounds__(256) k_inv_store(KParams P, TreeCoarse tc, con
             continue;
         }
         double v = A[(long long)row * ld + c];
-        if (tc.singular) {
-            const BlockDesc &o = P.B[tc.first + c / cells_of<D>(tc.n)];
-            const LevelDesc &L = P.L[o.lev];
-            double vol = L.vol;
-            if (P.geom == MG_CYL)
-                vol = 2.0 * M_PI * (P.lo[0] + (o.ijk[0] * tc.n + c % tc.n + 0.5) * L.h[0]) * L.h[0] * L.h[1];
-            v += vol / (sigma * vsum * vsum);
-        }
+        if (tc.singular) v += coarse_vol<D>(P, tc, c) / vsum / (coarse_shift(info, vsum) * vsum);
         minv[e] = v;
     }
 }
@@ -231,14 +247,14 @@ template <int D> static int inverse_d(mg_tree *t) {
                 const int x = B.ijk[0] * n + c % n, y = B.ijk[1] * n + c / n % n, z = D == 3 ? B.ijk[2] * n + c / (n * n) : 0;
                 map[((size_t)z * L.ncell[1] + y) * L.ncell[0] + x] = b * C + c;
             }
-        if (!calloc_dev((void **)&t->d_crow, sizeof(int) * map.size()) || !calloc_dev((void **)&t->d_cflag, sizeof(int)) ||
+        if (!calloc_dev((void **)&t->d_crow, sizeof(int) * map.size()) || !calloc_dev((void **)&t->d_cinfo, sizeof(CoarseInfo)) ||
             !calloc_dev((void **)&t->d_minv, sizeof(double) * (size_t)t->minv_total) ||
             !calloc_dev((void **)&t->d_cwork, sizeof(double) * ((size_t)nc * ld + 2 * (size_t)kPanel * ld)))
             return 1;
         if (cudaMemcpy(t->d_crow, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice) != cudaSuccess)
             return check_cuda("coarsest inverse");
     }
-    double vsum = 0, sigma = 0;
+    double vsum = 0;
     if (tc.singular) {
         for (int x = 0; x < L.ncell[0]; x++) {
             double V = 1.0;
@@ -246,30 +262,31 @@ template <int D> static int inverse_d(mg_tree *t) {
             if (t->geom == MG_CYL) V = 2.0 * M_PI * (t->lo[0] + (x + 0.5) * L.h[0]) * L.h[0] * L.h[1];
             vsum += V * L.ncell[1] * L.ncell[2];
         }
-        // the shift moves the constants' eigenvalue from 0 to - sigma v: to the size of 1 / h^2
-        double w = 0;
-        for (int d = 0; d < D; d++) w = std::max(w, 1.0 / (L.h[d] * L.h[d]));
-        sigma = w / vsum;
     }
     const KParams P = kparams(t, 1);
     double *A = t->d_cwork, *R = A + (size_t)nc * ld, *Cc = R + (size_t)kPanel * ld;
     cudaMemsetAsync(A, 0, sizeof(double) * (size_t)nc * ld, t->stream);
-    cudaMemsetAsync(t->d_cflag, 0, sizeof(int), t->stream);
+    cudaMemsetAsync(t->d_cinfo, 0, sizeof(CoarseInfo), t->stream);
     ++t->launches;
     launch_k(k_coarse_rows<D>, (nc + 127) / 128, 128, 0, t->stream, P, tc, (const int *)t->d_crow,
-             t->var_eps ? (const double *)t->f64.E : (const double *)nullptr, sigma, ld, A, t->d_cflag);
+             t->var_eps ? (const double *)t->f64.E : (const double *)nullptr, ld, A, t->d_cinfo);
+    const int elems = (int)std::max<long long>(1, std::min<long long>(((long long)nc * tc.ns + 255) / 256, 8LL * t->nsm));
+    if (tc.singular) {
+        ++t->launches;
+        launch_k(k_coarse_shift<D>, elems, 256, 0, t->stream, P, tc, ld, vsum, (const CoarseInfo *)t->d_cinfo, A);
+    }
     const int tiles = ld / kTile;
     for (int at = 0; at < nc; at += kPanel) {
         t->launches += 2;
-        launch_k(k_inv_panel, tiles, kPanelThreads, 0, t->stream, (const double *)A, nc, ld, at, R, Cc, t->d_cflag);
+        launch_k(k_inv_panel, tiles, kPanelThreads, 0, t->stream, (const double *)A, nc, ld, at, R, Cc, t->d_cinfo);
         launch_k(k_inv_update, dim3(tiles, tiles), kPanelThreads, 0, t->stream, A, nc, ld, at, (const double *)R,
                  (const double *)Cc);
     }
     ++t->launches;
-    launch_k(k_inv_store<D>, (int)std::max<long long>(1, std::min<long long>(((long long)nc * tc.ns + 255) / 256, 8LL * t->nsm)), 256, 0, t->stream, P, tc,
-             (const double *)A, ld, sigma, vsum, t->d_minv);
+    launch_k(k_inv_store<D>, elems, 256, 0, t->stream, P, tc, (const double *)A, ld, vsum,
+             (const CoarseInfo *)t->d_cinfo, t->d_minv);
     int flag = 0;
-    if (cudaMemcpyAsync(&flag, t->d_cflag, sizeof(int), cudaMemcpyDeviceToHost, t->stream) != cudaSuccess ||
+    if (cudaMemcpyAsync(&flag, &t->d_cinfo->flag, sizeof(int), cudaMemcpyDeviceToHost, t->stream) != cudaSuccess ||
         cudaStreamSynchronize(t->stream) != cudaSuccess)
         return check_cuda("coarsest inverse");
     const int rc = check_cuda("coarsest inverse");

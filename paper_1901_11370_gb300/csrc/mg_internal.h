@@ -171,6 +171,13 @@ struct LevelHost {
     std::vector<int> parents;  // segments holding the parents of its blocks
 };
 
+// Device words of the coarsest inverse (mg_coarse.cu)
+struct CoarseInfo {
+    unsigned long long amax;  // largest |diagonal|, the bits of the double
+    int flag;                 // 1: zero pivot, 2: eps not positive -- the host's pivoting inversion decides
+    int pad;
+};
+
 // Plan of the cluster kernel that runs the levels 0 .. top of a cycle
 // (mg_bottom.cu): the cut of each level into slabs, the shared-memory
 // layout of a CTA, and where the top level lives in the pool.
@@ -275,7 +282,8 @@ struct mg_tree {
     bool minv_ok = false;
     double *d_cvec = nullptr;      // coarsest residual vector (ns)
     double *d_cwork = nullptr;     // work of the device inverse (mg_coarse.cu)
-    int *d_crow = nullptr, *d_cflag = nullptr;  // its cell -> row map and status
+    int *d_crow = nullptr;         // its cell -> row map
+    mg::CoarseInfo *d_cinfo = nullptr;
     double *d_partials = nullptr;  // per-CTA norm partials (3 per CTA)
     int n_partials = 0;
     double *h_red = nullptr;       // reduced norms (3), pinned: the reductions write here
