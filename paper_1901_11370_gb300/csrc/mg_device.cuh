@@ -14,6 +14,7 @@
 namespace mg {
 
 static constexpr int kMaxThreads = 256;
+static constexpr size_t kMaxSmem = 227 * 1024;  // shared memory of a CTA, static and dynamic
 
 template <int D> __host__ __device__ constexpr int cells_of(int n) { return D == 2 ? n * n : n * n * n; }
 template <int D> __host__ __device__ constexpr int face_of(int n) { return D == 2 ? n : n * n; }

@@ -1419,7 +1419,9 @@ __global__ void __launch_bounds__(kMaxThreads) k_fas_rhs_vold(KParams P, int fir
 // cells under the block and their face halo: a cell then takes 4 FP64
 // instructions instead of 9 and four shared loads instead of eight global
 // ones (FP64 16^3 blocks, whose staged form does not fit: see prolong).
-template <class T, int D>
+// BOX false: blocks whose cells and box together exceed a CTA's shared memory
+// (2D FP64 from 152^2, FP32 from 216^2) form them per cell.
+template <class T, int D, bool BOX>
 __global__ void __launch_bounds__(kMaxThreads) k_prolong_push(KParams P, int first, Fields<T> F) {
     pdl_entry();
     __shared__ BlockDesc sb, sp;
@@ -1432,22 +1434,33 @@ __global__ void __launch_bounds__(kMaxThreads) k_prolong_push(KParams P, int fir
     const LevelDesc &L = P.L[b.lev];
     const int n = b.n, C = cells_of<D>(n), B = n / 2 + 2, BB = D == 3 ? B * B * B : B * B;
     T *box = xs + C;
-    for (int q = threadIdx.x; q < BB; q += blockDim.x) {
+    auto diff = [&](int i, int j, int k) { return load<T, D>(F.X, F.XG, p, i, j, k) - load<T, D>(F.V, F.VG, p, i, j, k); };
+    for (int q = threadIdx.x; BOX && q < BB; q += blockDim.x) {
         const int a = q % B, c = (q / B) % B, e = D == 3 ? q / (B * B) : 1;
         if ((a == 0 || a == B - 1) + (c == 0 || c == B - 1) + (D == 3 && (e == 0 || e == B - 1)) > 1) continue;  // never read
-        const int i = b.poff[0] + a - 1, j = b.poff[1] + c - 1, k = D == 3 ? b.poff[2] + e - 1 : 0;
-        box[q] = load<T, D>(F.X, F.XG, p, i, j, k) - load<T, D>(F.V, F.VG, p, i, j, k);
+        box[q] = diff(b.poff[0] + a - 1, b.poff[1] + c - 1, D == 3 ? b.poff[2] + e - 1 : 0);
     }
     __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x) {
         int i, j, k;
         cell_of(c, n, D, i, j, k);
         // blocks start at even cells: the local parity is the global one
-        const T *d = box + (D == 3 ? (k / 2 + 1) * B * B : 0) + (j / 2 + 1) * B + i / 2 + 1;
-        T nbs = d[(i & 1) ? 1 : -1];
-        nbs += d[(j & 1) ? B : -B];
-        if (D == 3) nbs += d[(k & 1) ? B * B : -B * B];
-        const T xn = F.X[b.cell_off + c] + (D == 2 ? (T)2 * d[0] + nbs : d[0] + nbs) * (T)0.25;
+        const int sx = (i & 1) ? 1 : -1, sy = (j & 1) ? 1 : -1, sz = (k & 1) ? 1 : -1;
+        T v0, nbs;
+        if (BOX) {
+            const T *d = box + (D == 3 ? (k / 2 + 1) * B * B : 0) + (j / 2 + 1) * B + i / 2 + 1;
+            v0 = d[0];
+            nbs = d[sx];
+            nbs += d[sy * B];
+            if (D == 3) nbs += d[sz * B * B];
+        } else {
+            const int ci = b.poff[0] + i / 2, cj = b.poff[1] + j / 2, ck = D == 3 ? b.poff[2] + k / 2 : 0;
+            v0 = diff(ci, cj, ck);
+            nbs = diff(ci + sx, cj, ck);
+            nbs += diff(ci, cj + sy, ck);
+            if (D == 3) nbs += diff(ci, cj, ck + sz);
+        }
+        const T xn = F.X[b.cell_off + c] + (D == 2 ? (T)2 * v0 + nbs : v0 + nbs) * (T)0.25;
         F.X[b.cell_off + c] = xn;
         xs[c] = xn;
     }
@@ -5223,9 +5236,11 @@ template <class T, int D> struct Launch {
             ghost(t, P, l, F.X, F.XG, 0);
             return;
         }
-        const size_t sm = sizeof(T) * (cells_of<D>(L.n) + cells_of<D>(L.n / 2 + 2));
-        set_smem(k_prolong_push<T, D>, sm);
-        launch_k(k_prolong_push<T, D>, L.nb, threads_for(cells_of<D>(L.n)), sm, t->stream, P, L.first, F);
+        const size_t cells = sizeof(T) * cells_of<D>(L.n), boxed = cells + sizeof(T) * cells_of<D>(L.n / 2 + 2);
+        const bool fits = boxed + 2 * sizeof(BlockDesc) <= kMaxSmem;  // the kernel's static part: two descriptors
+        auto kern = fits ? k_prolong_push<T, D, true> : k_prolong_push<T, D, false>;
+        set_smem(kern, fits ? boxed : cells);
+        launch_k(kern, L.nb, threads_for(cells_of<D>(L.n)), fits ? boxed : cells, t->stream, P, L.first, F);
     }
     // exact coarsest solves of the trees whose coarsest group is below `top`
     // (strict) or at most `top`; then ghost fills of the coarsest segments
