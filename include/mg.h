@@ -404,7 +404,9 @@ int mg_set_wait_limit(mg_tree *t, int64_t polls);
  * automatic choice).  MG_ERR_ARG when a single level is named and the
  * variant does not apply there.  Every variant computes the same red-black
  * half-sweep; this call exists to test and time them one by one.  While a
- * variant is pinned, solves run launch by launch on every level. */
+ * variant is pinned on a level that the solves' cluster kernel would run (see
+ * mg_solve), they run launch by launch on every level; a pin on a level above
+ * leaves the kernel on. */
 int mg_sweep_variant(mg_tree *t, int precision, int level, int *variant);
 int mg_set_sweep_variant(mg_tree *t, int precision, int level, int variant);
 /* mg_set_tail: an option for the small levels at the bottom of a V-cycle

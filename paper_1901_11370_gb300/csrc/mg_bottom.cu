@@ -1201,8 +1201,11 @@ template <class T> static void bot_coef_one(mg_tree *t, BotState &S, T *W, int t
 // current smoother, as bottom_prepare left it (cycles are enqueued inside
 // stream captures, so nothing is built here).
 template <class T> int bottom_level(mg_tree *t) {
-    if (!t->bottom_on || t->tail_cells > 0 || t->coarse_mode != MG_COARSE_EXACT || t->pinned[sizeof(T) == 4 ? 1 : 0]) return 0;
-    const BotState &S = t->bottom[sizeof(T) == 4 ? 1 : 0][t->smoother == MG_SMOOTH_JACOBI ? 1 : 0];
+    const int prec = sizeof(T) == 4 ? 1 : 0;
+    if (!t->bottom_on || t->tail_cells > 0 || t->coarse_mode != MG_COARSE_EXACT) return 0;
+    const BotState &S = t->bottom[prec][t->smoother == MG_SMOOTH_JACOBI ? 1 : 0];
+    for (int l = 0; l <= S.plan.top && l < (int)t->pinned[prec].size(); l++)
+        if (t->pinned[prec][l]) return 0;  // a pinned level runs its own sweeps
     return t->var_eps && !S.d_w ? 0 : S.plan.top;
 }
 

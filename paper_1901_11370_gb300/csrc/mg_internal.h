@@ -324,10 +324,10 @@ struct mg_tree {
     std::map<int, int> tune_hint[2];
     // cluster kernel of the lower levels (mg_bottom.cu): its plans per
     // precision and smoother; whether the running call uses it (the solve
-    // loops do); precisions whose sweep kernels the caller has pinned
+    // loops do); levels whose sweep kernel the caller has pinned, per precision
     mg::BotState bottom[2][2];
     bool bottom_on = false;
-    bool pinned[2] = {false, false};
+    std::vector<char> pinned[2];
 };
 
 namespace mg {

@@ -958,10 +958,15 @@ extern "C" int mg_tree_adapt(mg_tree *t, int n_add, const int32_t *add, int n_re
         for (const LevelHost &OL : t->lev)
             if (OL.depth == NL.depth && OL.n == NL.n)
                 for (int f = 0; f < 6; f++) NL.bc[f] = OL.bc[f];
-    // sweep kernels: the old tree's choices by depth, no second autotuning
-    for (int prec = 0; prec < 2; prec++)
+    // sweep kernels: the old tree's choices and pins by depth, no second autotuning
+    for (int prec = 0; prec < 2; prec++) {
         for (size_t l = 0; l < t->sweep_choice[prec].size() && l < t->lev.size(); l++)
             nt->tune_hint[prec][t->lev[l].depth] = t->sweep_choice[prec][l];
+        nt->pinned[prec].assign(nt->lev.size(), 0);
+        for (size_t l = 0; l < t->pinned[prec].size(); l++)
+            for (size_t m = 0; m < nt->lev.size(); m++)
+                if (t->pinned[prec][l] && nt->lev[m].depth == t->lev[l].depth) nt->pinned[prec][m] = 1;
+    }
     if ((rc = mg_tree_finalize(nt, t->stream))) {
         const std::string msg = mg_last_error();
         mg_tree_destroy(nt);
@@ -1651,15 +1656,17 @@ extern "C" int mg_set_sweep_variant(mg_tree *t, int precision, int level, int va
     if (precision == MG_FP32_DC && (rc = ensure_f32(t))) return rc;
     const int prec = precision == MG_FP32_DC ? 1 : 0;
     std::vector<int> &ch = t->sweep_choice[prec];
+    std::vector<char> &pin = t->pinned[prec];
     if (ch.size() != t->lev.size()) ch.assign(t->lev.size(), -1);
+    pin.resize(t->lev.size(), 0);
     if (level >= 0 && variant >= 0 && !sweep_variant_ok(t, prec, level, variant))
         return fail(MG_ERR_ARG, "sweep variant does not apply to this level");
     for (int l = 0; l < (int)t->lev.size(); l++) {
         if (level >= 0 && l != level) continue;
-        if (variant < 0) ch[l] = -1;
-        else if (sweep_variant_ok(t, prec, l, variant)) ch[l] = variant;
+        if (variant >= 0 && !sweep_variant_ok(t, prec, l, variant)) continue;
+        ch[l] = variant;
+        pin[l] = variant >= 0;
     }
-    t->pinned[prec] = variant >= 0 || (level >= 0 && t->pinned[prec]);  // pinned levels run their own sweeps
     drop_graphs(t);  // captured cycles hold the previous choice
     return MG_OK;
 }
