@@ -1146,7 +1146,7 @@ template <class T> static void bot_plan(mg_tree *t, bool jac, BotState &S) {
         }
     }
     if (cudaMalloc((void **)&S.d_map, sizeof(int) * map.size()) != cudaSuccess ||
-        cudaMemcpy(S.d_map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+        upload(S.d_map, map.data(), sizeof(int) * map.size(), t->stream) != cudaSuccess) {
         cudaGetLastError();
         B.top = 0;
         return;
@@ -1154,7 +1154,7 @@ template <class T> static void bot_plan(mg_tree *t, bool jac, BotState &S) {
     if (B.fd) {
         const std::vector<double> tab = fd_tables(t, B);
         if (cudaMalloc((void **)&S.d_fd, sizeof(double) * tab.size()) != cudaSuccess ||
-            cudaMemcpy(S.d_fd, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+            upload(S.d_fd, tab.data(), sizeof(double) * tab.size(), t->stream) != cudaSuccess) {
             cudaGetLastError();
             B.top = 0;
             return;

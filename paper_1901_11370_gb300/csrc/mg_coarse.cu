@@ -251,7 +251,7 @@ template <int D> static int inverse_d(mg_tree *t) {
             !calloc_dev((void **)&t->d_minv, sizeof(double) * (size_t)t->minv_total) ||
             !calloc_dev((void **)&t->d_cwork, sizeof(double) * ((size_t)nc * ld + 2 * (size_t)kPanel * ld)))
             return 1;
-        if (cudaMemcpy(t->d_crow, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        if (upload(t->d_crow, map.data(), sizeof(int) * map.size(), t->stream) != cudaSuccess)
             return check_cuda("coarsest inverse");
     }
     double vsum = 0;

@@ -13,6 +13,15 @@
 
 namespace mg {
 
+// Host to device on a stream, complete when it returns.  (cudaMemcpy from
+// pageable memory may return before its transfer ends, and the default stream
+// it runs on is not ordered with a stream that does not block on it.)
+inline cudaError_t upload(void *dst, const void *src, size_t bytes, cudaStream_t s) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+    const cudaError_t w = cudaStreamSynchronize(s);
+    return e != cudaSuccess ? e : w;
+}
+
 // polls of a bounded mbarrier wait before a kernel gives up, sets the status
 // word and returns (a few milliseconds)
 constexpr uint32_t kDefaultWaitLimit = 1u << 20;

@@ -6029,7 +6029,7 @@ extern "C" int mg_residual_norm_noalloc(mg_tree *t, double *l2, double *linf) {
         return MG_ERR_CUDA;
     }
     if (st) {
-        cudaMemset(t->d_status, 0, sizeof(int) * kStatusWords);
+        cudaMemsetAsync(t->d_status, 0, sizeof(int) * kStatusWords, t->stream);
         mg_set_error("a bounded wait in a residual kernel expired");
         return MG_ERR_TIMEOUT;
     }

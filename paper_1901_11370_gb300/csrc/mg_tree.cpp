@@ -449,19 +449,21 @@ extern "C" int mg_tree_leaf_blocks(mg_tree *t, int32_t *out) {
 
 // ------------------------------------------------ device allocation ----
 
-template <class T> static int dalloc(T **p, long long n) {
+// zeroed on the tree's stream: a fill on the default stream is not ordered
+// with a stream that does not block on it, and could come after first use
+template <class T> static int dalloc(mg_tree *t, T **p, long long n) {
     if (*p) return MG_OK;
     CK(cudaMalloc((void **)p, sizeof(T) * (size_t)std::max(1LL, n)));
-    CK(cudaMemset(*p, 0, sizeof(T) * (size_t)std::max(1LL, n)));
+    CK(cudaMemsetAsync(*p, 0, sizeof(T) * (size_t)std::max(1LL, n), t->stream));
     return MG_OK;
 }
 
 template <class T> static int alloc_fields(mg_tree *t, Fields<T> &F, bool with_eps) {
     int rc;
-    if ((rc = dalloc(&F.X, t->ncells)) || (rc = dalloc(&F.XG, t->nghost)) || (rc = dalloc(&F.F, t->ncells)) ||
-        (rc = dalloc(&F.V, t->ncells)) || (rc = dalloc(&F.VG, t->nghost)))
+    if ((rc = dalloc(t, &F.X, t->ncells)) || (rc = dalloc(t, &F.XG, t->nghost)) || (rc = dalloc(t, &F.F, t->ncells)) ||
+        (rc = dalloc(t, &F.V, t->ncells)) || (rc = dalloc(t, &F.VG, t->nghost)))
         return rc;
-    if (with_eps && ((rc = dalloc(&F.E, t->ncells)) || (rc = dalloc(&F.EG, t->nghost)))) return rc;
+    if (with_eps && ((rc = dalloc(t, &F.E, t->ncells)) || (rc = dalloc(t, &F.EG, t->nghost)))) return rc;
     return MG_OK;
 }
 
@@ -509,7 +511,7 @@ static int upload_bc(mg_tree *t) {
         }
     }
     if (!t->d_levels) CK(cudaMalloc((void **)&t->d_levels, sizeof(LevelDesc) * ld.size()));
-    CK(cudaMemcpy(t->d_levels, ld.data(), sizeof(LevelDesc) * ld.size(), cudaMemcpyHostToDevice));
+    CK(upload(t->d_levels, ld.data(), sizeof(LevelDesc) * ld.size(), t->stream));
     if ((long long)all.size() > t->n_bcplanes) {
         cudaFree(t->d_bcplanes);
         t->d_bcplanes = nullptr;
@@ -517,7 +519,7 @@ static int upload_bc(mg_tree *t) {
         t->n_bcplanes = (long long)all.size();
     }
     if (!all.empty())
-        CK(cudaMemcpy(t->d_bcplanes, all.data(), sizeof(double) * all.size(), cudaMemcpyHostToDevice));
+        CK(upload(t->d_bcplanes, all.data(), sizeof(double) * all.size(), t->stream));
     t->bc_dirty = false;
     return MG_OK;
 }
@@ -760,14 +762,14 @@ int build_coarse_inverse(mg_tree *t) {
     for (auto &e : errs)
         if (!e.empty()) return fail(MG_ERR_ARG, e);
     if (!t->d_minv) CK(cudaMalloc((void **)&t->d_minv, sizeof(double) * (size_t)std::max(1LL, t->minv_total)));
-    if (t->minv_total) CK(cudaMemcpy(t->d_minv, inv.data(), sizeof(double) * (size_t)t->minv_total, cudaMemcpyHostToDevice));
+    if (t->minv_total) CK(upload(t->d_minv, inv.data(), sizeof(double) * (size_t)t->minv_total, t->stream));
     if (t->bt_total) {
         if (!t->d_bt) CK(cudaMalloc((void **)&t->d_bt, sizeof(double) * (size_t)t->bt_total));
         if (!t->d_bt32) CK(cudaMalloc((void **)&t->d_bt32, sizeof(float) * (size_t)t->bt_total32));
         if (!t->d_btperm) CK(cudaMalloc((void **)&t->d_btperm, sizeof(int) * (size_t)t->btperm_total));
-        CK(cudaMemcpy(t->d_bt, bt.data(), sizeof(double) * (size_t)t->bt_total, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(t->d_bt32, bt32.data(), sizeof(float) * (size_t)t->bt_total32, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(t->d_btperm, perm.data(), sizeof(int) * (size_t)t->btperm_total, cudaMemcpyHostToDevice));
+        CK(upload(t->d_bt, bt.data(), sizeof(double) * (size_t)t->bt_total, t->stream));
+        CK(upload(t->d_bt32, bt32.data(), sizeof(float) * (size_t)t->bt_total32, t->stream));
+        CK(upload(t->d_btperm, perm.data(), sizeof(int) * (size_t)t->btperm_total, t->stream));
     }
     t->minv_ok = true;
     return MG_OK;
@@ -806,7 +808,7 @@ extern "C" int mg_tree_finalize(mg_tree *t, void *stream) {
         t->d_blocks_built = nullptr;
     } else {
         CK(cudaMalloc((void **)&t->d_blocks, sizeof(BlockDesc) * t->blocks.size()));
-        CK(cudaMemcpy(t->d_blocks, t->blocks.data(), sizeof(BlockDesc) * t->blocks.size(), cudaMemcpyHostToDevice));
+        CK(upload(t->d_blocks, t->blocks.data(), sizeof(BlockDesc) * t->blocks.size(), t->stream));
     }
     if ((rc = upload_bc(t))) return rc;
     if ((rc = alloc_fields(t, t->f64, false))) return rc;
@@ -814,11 +816,11 @@ extern "C" int mg_tree_finalize(mg_tree *t, void *stream) {
     long long nleafb = 0;
     for (auto &L : t->lev) { maxleaf = std::max(maxleaf, L.nb - L.nref); nleafb += L.nb - L.nref; }
     t->n_partials = (int)nleafb;
-    if ((rc = dalloc(&t->d_partials, 3 * nleafb))) return rc;
-    if ((rc = dalloc(&t->d_status, kStatusWords))) return rc;
-    if ((rc = dalloc(&t->d_cvec, t->cvec_total))) return rc;
+    if ((rc = dalloc(t, &t->d_partials, 3 * nleafb))) return rc;
+    if ((rc = dalloc(t, &t->d_status, kStatusWords))) return rc;
+    if ((rc = dalloc(t, &t->d_cvec, t->cvec_total))) return rc;
     CK(cudaMalloc((void **)&t->d_tcoarse, sizeof(TreeCoarse) * t->tcoarse.size()));
-    CK(cudaMemcpy(t->d_tcoarse, t->tcoarse.data(), sizeof(TreeCoarse) * t->tcoarse.size(), cudaMemcpyHostToDevice));
+    CK(upload(t->d_tcoarse, t->tcoarse.data(), sizeof(TreeCoarse) * t->tcoarse.size(), t->stream));
     {  // work lists of the coarse solve: kCoarseRows rows of one dense tree
        // per CTA; one CTA per block-tridiagonal tree
         std::vector<int2> ch;
@@ -845,20 +847,20 @@ extern "C" int mg_tree_finalize(mg_tree *t, void *stream) {
             for (int r = 0; r < t->tcoarse[i].nc; r += kBtResidCells) bc.push_back(make_int2(i, r));
         t->n_bt_chunks = (int)bc.size();
         CK(cudaMalloc((void **)&t->d_bt_chunks, sizeof(int2) * std::max<size_t>(1, bc.size())));
-        if (!bc.empty()) CK(cudaMemcpy(t->d_bt_chunks, bc.data(), sizeof(int2) * bc.size(), cudaMemcpyHostToDevice));
+        if (!bc.empty()) CK(upload(t->d_bt_chunks, bc.data(), sizeof(int2) * bc.size(), t->stream));
         t->n_coarse_chunks = (int)ch.size();
         t->n_btri = (int)bl.size();
         CK(cudaMalloc((void **)&t->d_coarse_chunks, sizeof(int2) * std::max<size_t>(1, ch.size())));
-        if (!ch.empty()) CK(cudaMemcpy(t->d_coarse_chunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice));
+        if (!ch.empty()) CK(upload(t->d_coarse_chunks, ch.data(), sizeof(int2) * ch.size(), t->stream));
         CK(cudaMalloc((void **)&t->d_btlist, sizeof(int) * std::max<size_t>(1, bl.size())));
-        if (!bl.empty()) CK(cudaMemcpy(t->d_btlist, bl.data(), sizeof(int) * bl.size(), cudaMemcpyHostToDevice));
+        if (!bl.empty()) CK(upload(t->d_btlist, bl.data(), sizeof(int) * bl.size(), t->stream));
     }
     CK(cudaMallocHost((void **)&t->h_red, 3 * sizeof(double)));
     CK(cudaStreamCreateWithFlags(&t->cap_stream, cudaStreamNonBlocking));
     t->finalized = true;
     if ((rc = build_coarse_inverse(t))) return rc;
     if (t->geom == MG_CYL) {  // r-face factors: precomputed FP64 face coefficients
-        if ((rc = dalloc(&t->d_wface, t->ncells * wstride(t->dim)))) return rc;
+        if ((rc = dalloc(t, &t->d_wface, t->ncells * wstride(t->dim)))) return rc;
         t->f64.W = t->d_wface;
         face_coef(t);
     }
@@ -1005,7 +1007,7 @@ static int check_status(mg_tree *t) {
     CK(cudaStreamSynchronize(t->stream));
     CK(cudaMemcpy(&st, t->d_status, sizeof(int), cudaMemcpyDeviceToHost));
     if (st) {
-        CK(cudaMemset(t->d_status, 0, sizeof(int) * kStatusWords));
+        CK(cudaMemsetAsync(t->d_status, 0, sizeof(int) * kStatusWords, t->stream));
         return fail(MG_ERR_TIMEOUT, "a bounded wait in a kernel expired");
     }
     return MG_OK;
@@ -1136,7 +1138,7 @@ extern "C" int mg_set_eps(mg_tree *t, const double *e) {
     NEED_FINAL(t);
     if (!e) return fail(MG_ERR_ARG, "null eps");
     int rc;
-    if ((rc = dalloc(&t->f64.E, t->ncells)) || (rc = dalloc(&t->f64.EG, t->nghost))) return rc;
+    if ((rc = dalloc(t, &t->f64.E, t->ncells)) || (rc = dalloc(t, &t->f64.EG, t->nghost))) return rc;
     if (!t->var_eps) {  // eps pointers enter the captured kernels; the cluster kernel's coarsest solve changes
         drop_graphs(t);
         bottom_free(t);
@@ -1144,7 +1146,7 @@ extern "C" int mg_set_eps(mg_tree *t, const double *e) {
     t->var_eps = true;
     if ((rc = leaf_copy(t, t->f64.E, e, true))) return rc;
     refresh_eps<double>(t, t->f64);
-    if ((rc = dalloc(&t->d_wface, t->ncells * wstride(t->dim)))) return rc;
+    if ((rc = dalloc(t, &t->d_wface, t->ncells * wstride(t->dim)))) return rc;
     t->f64.W = t->d_wface;  // precomputed FP64 face coefficients for the residual
     face_coef(t);
     t->adj.E = t->f64.E;
@@ -1152,7 +1154,7 @@ extern "C" int mg_set_eps(mg_tree *t, const double *e) {
     t->adj.EG = t->f64.EG;
     bottom_coef(t);
     if (t->f32.X) {
-        if ((rc = dalloc(&t->f32.E, t->ncells)) || (rc = dalloc(&t->f32.EG, t->nghost))) return rc;
+        if ((rc = dalloc(t, &t->f32.E, t->ncells)) || (rc = dalloc(t, &t->f32.EG, t->nghost))) return rc;
         copy_eps_to_f32(t);
     }
     if ((rc = check_cuda("set_eps"))) return rc;
@@ -1208,10 +1210,10 @@ static int use_params(mg_tree *t, const mg_params *p, mg_params *q, std::string 
     t->coarse_rel = q->coarse_rel_tol;
     int rc;
     if (q->smoother == MG_SMOOTH_JACOBI) {
-        if ((rc = dalloc(&t->d_jac64, t->ncells))) return rc;
+        if ((rc = dalloc(t, &t->d_jac64, t->ncells))) return rc;
         t->f64.J = t->adj.J = t->d_jac64;
         if (q->precision == MG_FP32_DC) {
-            if ((rc = dalloc(&t->d_jac32, t->ncells))) return rc;
+            if ((rc = dalloc(t, &t->d_jac32, t->ncells))) return rc;
             t->f32.J = t->d_jac32;
         }
     }
@@ -1300,7 +1302,7 @@ extern "C" int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_firs
     if (t->singular && !t->is_batch) {
         // no Dirichlet face and lambda = 0: the weighted mean of the residual
         // does not change with phi, so its size bounds what cycles can reach
-        if ((rc = dalloc(&t->d_r64, t->nleaf_cells))) return rc;
+        if ((rc = dalloc(t, &t->d_r64, t->nleaf_cells))) return rc;
         residual_norm(t, t->f64, 0, o, t->d_r64, nullptr);
         const double l2 = std::sqrt(o[0] / o[1]), mean = std::fabs(leaf_mean(t, t->d_r64));
         if ((rc = check_cuda("compatibility")) != MG_OK) return rc;
@@ -1374,7 +1376,7 @@ extern "C" int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_firs
         // no Dirichlet face: phi is fixed up to a constant; return the
         // solution with zero volume-weighted mean (covered cells and ghosts
         // shift with it)
-        if ((rc = dalloc(&t->d_r64, t->nleaf_cells)) || (rc = leaf_copy(t, t->f64.X, (const double *)t->d_r64, false)))
+        if ((rc = dalloc(t, &t->d_r64, t->nleaf_cells)) || (rc = leaf_copy(t, t->f64.X, (const double *)t->d_r64, false)))
             return rc;
         const double mean = leaf_mean(t, t->d_r64);
         sub_scalar(t, t->f64.X, mean, t->ncells);
@@ -1713,7 +1715,7 @@ extern "C" int mg_clean(mg_tree *t, const double *B, double *Bnew, double *divB,
     NEED_FINAL(t);
     if (!B || !Bnew) return fail(MG_ERR_ARG, "null argument");
     int rc;
-    if ((rc = dalloc(&t->d_r64, t->nleaf_cells))) return rc;
+    if ((rc = dalloc(t, &t->d_r64, t->nleaf_cells))) return rc;
     if ((rc = mg_divergence_order(t, B, t->d_r64, order))) return rc;
     if (t->singular) sub_scalar(t, t->d_r64, leaf_mean(t, t->d_r64), t->nleaf_cells);
     if (divB) CK(cudaMemcpyAsync(divB, t->d_r64, sizeof(double) * t->nleaf_cells, cudaMemcpyDeviceToDevice, t->stream));
@@ -1942,7 +1944,7 @@ static int batch_device_tables(mg_tree *P, int n) {
         }
     P->n_runs = (int)(runs.size() / 3);
     CK(cudaMalloc((void **)&P->d_runs, sizeof(long long) * std::max<size_t>(3, runs.size())));
-    if (!runs.empty()) CK(cudaMemcpy(P->d_runs, runs.data(), sizeof(long long) * runs.size(), cudaMemcpyHostToDevice));
+    if (!runs.empty()) CK(upload(P->d_runs, runs.data(), sizeof(long long) * runs.size(), P->stream));
     // residual slots: one per leaf block, in the order the residual pass
     // visits them (segments in order, leaf blocks in order), listed per tree
     std::vector<std::vector<int>> per(n);
@@ -1965,9 +1967,9 @@ static int batch_device_tables(mg_tree *P, int n) {
         slots.insert(slots.end(), per[i].begin(), per[i].end());
     }
     CK(cudaMalloc((void **)&P->d_slot_off, sizeof(int) * (n + 1)));
-    CK(cudaMemcpy(P->d_slot_off, off.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice));
+    CK(upload(P->d_slot_off, off.data(), sizeof(int) * (n + 1), P->stream));
     CK(cudaMalloc((void **)&P->d_slots, sizeof(int) * std::max<size_t>(1, slots.size())));
-    if (!slots.empty()) CK(cudaMemcpy(P->d_slots, slots.data(), sizeof(int) * slots.size(), cudaMemcpyHostToDevice));
+    if (!slots.empty()) CK(upload(P->d_slots, slots.data(), sizeof(int) * slots.size(), P->stream));
     CK(cudaMalloc((void **)&P->d_tree3, sizeof(double) * 3 * n));
     CK(cudaMallocHost((void **)&P->h_tree3, sizeof(double) * 3 * n));
     return MG_OK;
