@@ -293,9 +293,22 @@ template <int D> static int inverse_d(mg_tree *t) {
     return rc ? rc : (flag ? 1 : 0);  // zero pivot or eps <= 0: the host's pivoting inversion decides
 }
 
+void coarse_inverse_free(mg_tree *t) {
+    cudaFree(t->d_cwork);
+    cudaFree(t->d_crow);
+    cudaFree(t->d_cinfo);
+    t->d_cwork = nullptr;
+    t->d_crow = nullptr;
+    t->d_cinfo = nullptr;
+}
+
+// The scratch (as large as the inverse) stays while eps may be set again; a
+// constant coefficient is inverted once, when the tree is made.
 int coarse_inverse_device(mg_tree *t) {
     if (t->is_batch || t->tcoarse.size() != 1 || t->tcoarse[0].bt_n) return 1;
-    return t->dim == 2 ? inverse_d<2>(t) : inverse_d<3>(t);
+    const int rc = t->dim == 2 ? inverse_d<2>(t) : inverse_d<3>(t);
+    if (!t->var_eps || rc > 0) coarse_inverse_free(t);
+    return rc;
 }
 
 }  // namespace mg

@@ -384,6 +384,7 @@ KParams kparams(mg_tree *t, int homog);
 // dense inverse of a single tree's coarsest level on the device (mg_coarse.cu):
 // 0 done, 1 left to the host, < 0 an error
 int coarse_inverse_device(mg_tree *t);
+void coarse_inverse_free(mg_tree *t);
 // the lower levels in one launch (mg_bottom.cu)
 template <class T> int bottom_level(mg_tree *t);
 template <class T> void bottom_prepare(mg_tree *t);
