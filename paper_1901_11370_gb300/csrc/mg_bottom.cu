@@ -935,6 +935,22 @@ __global__ void __launch_bounds__(256) k_bottom_coef(BotPlan B, int l, const int
     }
 }
 
+// The inverses along p of the eigenvector solve, [p'][p][kb][ka]: one sum over
+// the NP modes per value.  On the device because the sums are plane NP^3: 32 s
+// on one host core for a coarsest level of 3 x 1800 cells.
+__global__ void __launch_bounds__(256) k_fd_table(const double *__restrict__ Q, const double *__restrict__ w, int plane,
+                                                  int NP, double *__restrict__ out) {
+    pdl_entry();
+    const long long total = (long long)plane * NP * NP;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const int kab = (int)(e % plane), s = (int)(e / plane % NP), p = (int)(e / plane / NP);
+        double v = 0;
+        for (int k = 0; k < NP; k++)
+            v = fma(Q[(long long)k * NP + p] * w[(long long)k * plane + kab], Q[(long long)k * NP + s], v);
+        out[e] = v;
+    }
+}
+
 // ------------------------------------------------------------ host side ---
 
 template <class T, int D, bool VAR> static int bot_clusters(int cs, size_t smem) {
@@ -1063,11 +1079,11 @@ static void line_modes(int n, double h, int lo, int hi, std::vector<double> &Q, 
     }
 }
 
-// Tables of the eigenvector solve of the coarsest level (coarse_fd): the
-// modes along a and b, then per (ka, kb) the inverse along p,
+// Tables of the eigenvector solve of the coarsest level (coarse_fd) into
+// S.d_fd: the modes along a and b, then per (ka, kb) the inverse along p,
 // Q_p diag(-1 / (lam_a + lam_b + lam_p + lambda)) Q_p^T, as [p'][p][kb][ka].
-// The constants of a singular problem get 0.
-static std::vector<double> fd_tables(const mg_tree *t, const BotPlan &B) {
+// The constants of a singular problem get 0.  False: no memory.
+static bool fd_tables(mg_tree *t, const BotPlan &B, BotState &S) {
     const LevelHost &L = t->lev[0];
     std::vector<double> Q[3], lam[3];
     for (int i = 0; i < 3; i++) {
@@ -1079,26 +1095,34 @@ static std::vector<double> fd_tables(const mg_tree *t, const BotPlan &B) {
         }
         line_modes(L.ncell[d], L.h[d], t->bc.type[2 * d], t->bc.type[2 * d + 1], Q[i], lam[i]);
     }
-    std::vector<double> out(Q[0]);
-    if (t->dim == 3) out.insert(out.end(), Q[1].begin(), Q[1].end());
-    const int A = B.n0[0], NB = t->dim == 3 ? B.n0[1] : 1, NP = B.n0[2];
-    const size_t g0 = out.size(), plane = (size_t)A * NB;
-    out.resize(g0 + plane * NP * NP);
-    for (int kb = 0; kb < NB; kb++)
-        for (int ka = 0; ka < A; ka++) {
-            std::vector<double> w(NP);
-            for (int k = 0; k < NP; k++) {
+    std::vector<double> head(Q[0]);
+    if (t->dim == 3) head.insert(head.end(), Q[1].begin(), Q[1].end());
+    const size_t A = B.n0[0], NB = t->dim == 3 ? B.n0[1] : 1, NP = B.n0[2], plane = A * NB;
+    // the sums along p run on the device: modes [k][p], then weights [k][kb][ka]
+    std::vector<double> in(NP * NP + NP * plane);
+    for (size_t k = 0; k < NP; k++) {
+        for (size_t p = 0; p < NP; p++) in[k * NP + p] = Q[2][p * NP + k];
+        for (size_t kb = 0; kb < NB; kb++)
+            for (size_t ka = 0; ka < A; ka++) {
                 const bool constant = t->singular && ka == 0 && kb == 0 && k == 0;
-                w[k] = constant ? 0.0 : -1.0 / (lam[0][ka] + lam[1][kb] + lam[2][k] + t->helm);
+                in[NP * NP + (k * NB + kb) * A + ka] = constant ? 0.0 : -1.0 / (lam[0][ka] + lam[1][kb] + lam[2][k] + t->helm);
             }
-            for (int p = 0; p < NP; p++)
-                for (int s = 0; s < NP; s++) {
-                    double v = 0;
-                    for (int k = 0; k < NP; k++) v += Q[2][(size_t)p * NP + k] * w[k] * Q[2][(size_t)s * NP + k];
-                    out[g0 + ((size_t)p * NP + s) * plane + (size_t)kb * A + ka] = v;
-                }
-        }
-    return out;
+    }
+    const size_t total = plane * NP * NP;
+    double *d_in = nullptr;
+    bool ok = cudaMalloc((void **)&S.d_fd, sizeof(double) * (head.size() + total)) == cudaSuccess &&
+              cudaMalloc((void **)&d_in, sizeof(double) * in.size()) == cudaSuccess &&
+              upload(S.d_fd, head.data(), sizeof(double) * head.size(), t->stream) == cudaSuccess &&
+              upload(d_in, in.data(), sizeof(double) * in.size(), t->stream) == cudaSuccess;
+    if (ok) {
+        ++t->launches;
+        launch_k(k_fd_table, (int)std::min<size_t>((total + 255) / 256, 32 * (size_t)t->nsm), 256, 0, t->stream,
+                 (const double *)d_in, (const double *)(d_in + NP * NP), (int)plane, (int)NP, S.d_fd + head.size());
+        ok = cudaStreamSynchronize(t->stream) == cudaSuccess;
+    }
+    cudaFree(d_in);
+    if (!ok) cudaGetLastError();
+    return ok;
 }
 
 template <class T> static void bot_plan(mg_tree *t, bool jac, BotState &S) {
@@ -1152,10 +1176,7 @@ template <class T> static void bot_plan(mg_tree *t, bool jac, BotState &S) {
         return;
     }
     if (B.fd) {
-        const std::vector<double> tab = fd_tables(t, B);
-        if (cudaMalloc((void **)&S.d_fd, sizeof(double) * tab.size()) != cudaSuccess ||
-            upload(S.d_fd, tab.data(), sizeof(double) * tab.size(), t->stream) != cudaSuccess) {
-            cudaGetLastError();
+        if (!fd_tables(t, B, S)) {
             B.top = 0;
             return;
         }
