@@ -237,9 +237,15 @@ int mg_residual_norm(mg_tree *t, double *l2, double *linf, double *dev_r);
  * and adds e to phi in FP64.  *cycles_done counts outer steps, *rel_out the
  * final relative residual.  On a singular problem phi is returned with zero
  * volume-weighted mean.  Returns MG_ERR_NOT_CONVERGED at max_cycles.
- * On a single Cartesian tree the levels below the base grid (and small base
- * grids) run in one thread-block-cluster launch per cycle leg, the same
- * cycle up to rounding order; mg_vcycle and mg_fmg run launch by launch.
+ * On a single Cartesian tree of at least two levels the lowest levels run in
+ * one thread-block-cluster launch per cycle leg, the same cycle up to rounding
+ * order: level 0 up to the largest that covers the domain (the base grid at
+ * most), holds at most 40,000 cells (100,000 in 2D FP32 cycles) and fits the
+ * cluster's shared memory with all levels below it.  So do the other calls
+ * that solve: mg_adjoint, mg_adjoint_solve, mg_clean, mg_clean_adjoint,
+ * mg_tune_schedule.  Launch by launch on every level: MG_COARSE_SMOOTH, the
+ * tail option (mg_set_tail), a sweep variant pinned on one of these levels
+ * (mg_set_sweep_variant), batches, and the single cycles mg_vcycle and mg_fmg.
  */
 int mg_solve(mg_tree *t, double rel_tol, int max_cycles, int fmg_first,
              const mg_params *p, int *cycles_done, double *rel_out);
@@ -390,7 +396,8 @@ int mg_launch_count(mg_tree *t, int64_t *n);
  * path: no solve is meaningful until the limit is restored. */
 int mg_set_wait_limit(mg_tree *t, int64_t polls);
 /* mg_sweep_variant: the sweep kernel variant in use for a level and
- * precision (MG_FP64 / MG_FP32_DC): 0 persistent CTA-per-block TMA,
+ * precision (MG_FP64 / MG_FP32_DC): 0 persistent CTA-per-block TMA
+ * (3D 16^3 blocks in FP32: quarter rows, three stages),
  * 1 CTA-per-block plain loads, 2 / 3 warp-per-block TMA (8 / 4 warps),
  * 4 / 5 row-wise warp TMA (8 warps x 2 stages / 4 warps x 3 stages),
  * 6 one thread per colour cell (blocks of at most 16 cells without

@@ -990,7 +990,7 @@ template <class T> static size_t bot_layout(const mg_tree *t, BotPlan &B, int to
     // by eigenvectors from 400 cells on: 7.7 against 26 us for 36 x 27 cells,
     // 13 against 14 for 8^3; below, its five dependent FP64 stages take longer
     // than the rows of the inverse (8.0 against 6.1 for 180 cells, 5.6 against
-    // 3.7 for 8 x 8)
+    // 3.7 for 8 x 8).  Nothing between 180 and 512 cells was measured.
     B.fd = !t->var_eps && t->nc >= 400 && tab <= 2600;
     const long long plane = (long long)B.n0[0] * (D == 3 ? B.n0[1] : 1);
     const long long scratch = B.fd ? tab + (2 * B.mp + B.n0[2]) * plane : t->ns;
@@ -1137,7 +1137,8 @@ template <class T> static void bot_plan(mg_tree *t, bool jac, BotState &S) {
     // and 67 ms on the 256^3 variable-coefficient problem.  2D has smaller
     // faces: 62k cells 1.66 ms, 15k cells 1.81 ms, launch by launch 2.74.
     // FP64 32^3 against 16^3 as top level: 15.8 and 17.2 ms (128^3 Jacobi),
-    // 7.4 and 9.7 ms (64^3 cleaning with its adjoint).
+    // 7.4 and 9.7 ms (64^3 cleaning with its adjoint).  2D FP64 takes the 3D
+    // limit unmeasured.
     const long long limit = sizeof(T) == 4 && t->dim == 2 ? 100000 : 40000;
     for (int cs : {16, 8, 4, 2, 1}) {
         BotPlan B{};

@@ -4920,8 +4920,9 @@ template <class T, int D> struct Launch {
                     return;
                 }
             }
-            auto kern = n == 8 ? (half ? k_sweep_tma<T, D, 8, true> : k_sweep_tma<T, D, 8>)
-                               : (half || rows16() ? k_sweep_tma<T, D, 16, true> : k_sweep_tma<T, D, 16, rows16()>);
+            auto kern = n == 16 ? k_sweep_tma<T, D, 16, true> : (half ? k_sweep_tma<T, D, 8, true> : k_sweep_tma<T, D, 8>);
+            if constexpr (!rows16())  // (there the full-width form of 16^3 blocks is the one above)
+                if (n == 16 && !half) kern = k_sweep_tma<T, D, 16>;
             const int thr = sweep_tma_threads(cells_of<D>(n) / 2, half);
             const int grid = std::min(nb, resident_ctas(kern, thr, sm) * t->nsm);
             launch_k(kern, grid, thr, sm, t->stream, P, L.first, nb, F, colour);

@@ -1225,9 +1225,9 @@ static int use_params(mg_tree *t, const mg_params *p, mg_params *q, std::string 
     return MG_OK;
 }
 
-// The solve loops run the lower levels in one cluster launch per cycle;
-// mg_vcycle and mg_fmg keep the launch-by-launch cycle, which the sweep
-// variants and the tail option are defined on.
+// The solve loops run the lower levels in one cluster launch per cycle leg;
+// mg_vcycle and mg_fmg still run launch by launch, the form that the tests
+// compare the cluster kernel with.
 struct BottomScope {
     mg_tree *t;
     bool was;
