@@ -241,7 +241,8 @@ int mg_residual_norm(mg_tree *t, double *l2, double *linf, double *dev_r);
  * one thread-block-cluster launch per cycle leg, the same cycle up to rounding
  * order: level 0 up to the largest that covers the domain (the base grid at
  * most), holds at most 40,000 cells (100,000 in 2D FP32 cycles) and fits the
- * cluster's shared memory with all levels below it.  So do the other calls
+ * cluster's shared memory with all levels below it, where the coarsest solve
+ * is small enough (2048 cells with the dense inverse).  So do the other calls
  * that solve: mg_adjoint, mg_adjoint_solve, mg_clean, mg_clean_adjoint,
  * mg_tune_schedule.  Launch by launch on every level: MG_COARSE_SMOOTH, the
  * tail option (mg_set_tail), a sweep variant pinned on one of these levels

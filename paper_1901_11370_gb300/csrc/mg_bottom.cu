@@ -992,6 +992,13 @@ template <class T> static size_t bot_layout(const mg_tree *t, BotPlan &B, int to
     // than the rows of the inverse (8.0 against 6.1 for 180 cells, 5.6 against
     // 3.7 for 8 x 8).  Nothing between 180 and 512 cells was measured.
     B.fd = !t->var_eps && t->nc >= 400 && tab <= 2600;
+    // The coarsest solve reads the inverse (nc^2 values) or the tables along p
+    // (nc n_p) through 16 SMs.  Above 2048^2 values that takes longer than the
+    // whole chip needs, launches and all, for every level of the cycle: 4
+    // V-cycles with a dense inverse of 1800 cells 461 against 526 us, 2520
+    // 833 / 790, 3348 1063 / 765, 5400 2250 / 1016; with tables of 3500 x 70
+    // values 312 / 585, of 5400 x 1800 1094 / 742.
+    if ((long long)t->nc * (B.fd ? B.n0[2] : t->nc) > 2048LL * 2048) return 0;
     const long long plane = (long long)B.n0[0] * (D == 3 ? B.n0[1] : 1);
     const long long scratch = B.fd ? tab + (2 * B.mp + B.n0[2]) * plane : t->ns;
     const size_t head = sizeof(double) * (size_t)(16 + scratch);

@@ -59,3 +59,30 @@ def test_pins_and_the_cluster_kernel(mg, precision):
     b.set_rhs(za + 1.0)
     launches(b, za)
     assert launches(b, za) > free
+
+
+@pytest.mark.parametrize("cells, eps, cluster", [((200, 120), True, True), ((248, 216), True, False),
+                                                 ((248, 216), False, False), ((200, 280), False, True)])
+def test_a_large_coarsest_solve_stays_with_the_whole_chip(mg, cells, eps, cluster):
+    """Coarsest levels of 1500 and 3348 cells with the dense inverse (the
+    second cannot take eigenvectors), of 3500 with eigenvectors: whether the
+    solves take the cluster kernel, by what a pin on its levels changes."""
+    import torch
+    p = W.Problem("box", 2, 4, 0, cells + (1,), (0.0,) * 3, (1.0,) * 3, (0, 1, 0, 1, 2, 2), (0.0,) * 6,
+                  np.zeros((0, 4), np.int32), 4000)
+    t = mg.Tree.from_problem(p)
+    assert t.levels()[0]["ncell"][:2] == (cells[0] // 4, cells[1] // 4)
+    one = torch.ones(t.n_leaf, dtype=torch.float64, device="cuda")
+    t.set_rhs(one)
+    if eps:
+        t.set_eps(2 * one)
+    n = []
+    for pin in (False, True):
+        if pin:
+            t.set_sweep_variant(1, level=1)
+        for _ in range(2):
+            t.set_phi(0 * one)
+            n0 = t.launch_count()
+            t.solve(1e-30, 2, raise_on_fail=False)
+        n.append(t.launch_count() - n0)
+    assert (n[0] < n[1]) == cluster, n
