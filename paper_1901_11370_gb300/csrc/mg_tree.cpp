@@ -709,7 +709,7 @@ static void coarse_plan(const mg_tree *src, TreeCoarse &tc, const LevelHost &L, 
 }
 
 // Coarsest-level factors: a single tree's dense inverse on the device
-// (mg_coarse.cu); else of every tree (trees in parallel host threads):
+// (mg_coarse.cu) where that is sooner; else of every tree (trees in parallel host threads):
 // dense inverses, and plane records of the block-tridiagonal trees.
 int build_coarse_inverse(mg_tree *t) {
     const int dev = coarse_inverse_device(t);
@@ -717,11 +717,12 @@ int build_coarse_inverse(mg_tree *t) {
         t->minv_ok = dev == 0;
         return dev;
     }
-    std::vector<double> eps;
+    std::vector<double> eps;  // of the coarsest level; a batch's levels lie scattered: all of it
+    const long long e0 = t->is_batch ? 0 : t->tcoarse[0].cell0, ne = t->is_batch ? t->ncells : t->tcoarse[0].nc;
     if (t->var_eps) {
         CK(cudaStreamSynchronize(t->stream));
-        eps.resize(t->ncells);
-        CK(cudaMemcpy(eps.data(), t->f64.E, sizeof(double) * t->ncells, cudaMemcpyDeviceToHost));
+        eps.resize(ne);
+        CK(cudaMemcpy(eps.data(), t->f64.E + e0, sizeof(double) * ne, cudaMemcpyDeviceToHost));
     }
     std::vector<double> inv(t->minv_total), bt(t->bt_total);
     std::vector<float> bt32(t->bt_total32);
@@ -733,7 +734,7 @@ int build_coarse_inverse(mg_tree *t) {
         for (int i = next++; i < (int)t->tcoarse.size(); i = next++) {
             const TreeCoarse &tc = t->tcoarse[i];
             const LevelHost &L = t->is_batch ? t->tl[tc.lvl] : t->lev[tc.lvl];
-            const double *e = t->var_eps ? eps.data() + tc.cell0 : nullptr;
+            const double *e = t->var_eps ? eps.data() + (tc.cell0 - e0) : nullptr;
             if (!tc.bt_n) {
                 errs[i] = coarse_inverse_one(t, tc, L, e, inv.data() + tc.minv_off);
                 continue;
